@@ -41,9 +41,13 @@
  *                         2^-16 relative (mid.mid, hi.lo, lo.hi, hi.mid,
  *                         mid.hi, hi.hi), so every term keeps about FP32
  *                         precision; about half the rate of SPLIT_BF16X3.
- *                         SPLIT_BF16X3 itself takes this form for inner
- *                         dimensions m < 2237, where two parts cannot meet its
- *                         tolerance.  Not in the paper.
+ *                         For inner dimensions m < 2237, where two bf16 parts
+ *                         cannot meet its tolerance, SPLIT_BF16X3 itself splits
+ *                         every operand, scaled by one power of two, into two
+ *                         fp16 parts (three products, each term within about
+ *                         2^-21) where the operands' magnitudes fit fp16, and
+ *                         takes this form where they do not (a device-side
+ *                         choice from the data).  Not in the paper.
  *   MM_MODE_AUTO          SPLIT_BF16X3 for MM_F32, DGEMM for MM_F64.
  *   MM_MODE_OZAKI         FP64 in/out on the e4m3 tensor cores (Ozaki
  *                         scheme): each row of A / column of B is scaled by a

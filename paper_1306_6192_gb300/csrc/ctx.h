@@ -98,7 +98,9 @@ mm_status note_cuda(cudaError_t e);
 
 // Kind of split used for inner dimension m: two bf16 parts (three products)
 // where their worst-case per-product error 3 * 2^-16 is within the stated
-// tolerance 1e-6 sqrt(m), three parts (six products) below that.
+// tolerance 1e-6 sqrt(m); below that two fp16 parts (three products, at most
+// 2^-21 per product) where the magnitudes allow them, else three bf16 parts
+// (six products).
 TcKind split_kind_for(int64_t m);
 // The kind a split-path mode runs with for inner dimension m.
 inline TcKind split_kind_of(mm_mode mode, int64_t m) {
@@ -111,7 +113,7 @@ inline TcKind split_kind_of(mm_mode mode, int64_t m) {
 // dimensions only) always takes bn = 128: its 128-wide layout keeps a
 // four-stage ring beside the epilogue's staging buffers.
 inline int tc_bn(TcKind kind, int bn) {
-  if (kind == kTcSplitBf16x6) return 128;
+  if (kind == kTcSplitBf16x6 || kind == kTcSplitF16x3) return 128;
   return (bn == 64 && pack_parts(kind) != 2) ? 128 : bn;
 }
 

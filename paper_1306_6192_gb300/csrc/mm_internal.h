@@ -31,7 +31,11 @@ constexpr int kTcBM = 128;
 constexpr int kPackRowBytes = 128;
 // Split kinds: two bf16 parts (hi, lo; products hi.hi + hi.lo + lo.hi) or
 // three (hi, mid, lo; the six products down to 2^-16 relative).
-enum TcKind : int { kTcSplitBf16x3 = 0, kTcE4m3 = 1, kTcSplitBf16x6 = 2 };
+// kTcSplitF16x3: two fp16 parts (hi and 2^11 lo, three products) where the
+// operands' magnitudes allow it, decided per product on the device; a product
+// they do not allow takes the three bf16 parts, so its pack region has room
+// for three.
+enum TcKind : int { kTcSplitBf16x3 = 0, kTcE4m3 = 1, kTcSplitBf16x6 = 2, kTcSplitF16x3 = 3 };
 // elements per pack row and operand parts
 inline int pack_k(TcKind k) { return k == kTcE4m3 ? 128 : 64; }
 inline int pack_parts(TcKind k) { return k == kTcE4m3 ? 1 : (k == kTcSplitBf16x3 ? 2 : 3); }
@@ -122,9 +126,23 @@ struct SplitProb {
   // 1 + index of C's tensor map in the launch's map array (tiled stores of
   // the epilogue); 0: C is written with plain stores
   int32_t c_tma;
+  // kTcSplitF16x3: the product's state words (HalfState) on the device
+  int32_t *hx;
   // C = alpha (A.B) + beta D (plain stores only; off: C = A.B)
   EpiF epi;
 };
+
+// State words of a kTcSplitF16x3 product (SplitProb::hx), written on the
+// device before its pack.  kHalfX6: the sampled magnitudes do not fit the fp16
+// parts, so the product is packed as three bf16 parts; kHalfExpA / kHalfExpB:
+// the power of two 2^e that multiplies every entry of A / B before the fp16
+// split; kHalfBad: set by the pack where an entry falls outside the fp16
+// window (the product is then packed again as three bf16 parts).
+enum HalfState : int { kHalfX6 = 0, kHalfExpA = 1, kHalfExpB = 2, kHalfBad = 3, kHalfWords = 4 };
+
+// Counters per split tile of the kTcSplitF16x3 kind: one per
+// epilogue warp of its kernel, whose blocks are counted each on its own.
+constexpr int kHalfSplitCnt = 8;
 
 // Work units of a product with its tail split: whole tiles, then the parts.
 __host__ __device__ inline int64_t split_units(const SplitProb &sp) {
@@ -199,6 +217,7 @@ cudaError_t launch_simt_splitk_f64(int64_t n, int64_t m, int64_t p, const double
 // of range.
 // `map` arguments: item -> problem index arrays written by
 // launch_split_maps for tables of several problems, or nullptr.
+// Also writes the state words of kTcSplitF16x3 products (SplitProb::hx).
 cudaError_t launch_split_maps(const SplitProb *d_probs, int nprobs, int *unit_map,
                               int *pack_map, int *ver_map, cudaStream_t s);
 // Verify items of a product: 32 rows/columns each.
@@ -210,7 +229,7 @@ constexpr int kFlagScaleA = 1, kFlagScaleB = 2;
 // returns at once unless *any is set, then re-packs the tiles of flagged
 // operands (flags[g]).
 cudaError_t launch_split_pack(TcKind kind, int mode, const SplitProb *d_probs, int nprobs,
-                              int total_tiles, const int *map, const int *flags, const int *any,
+                              int total_tiles, const int *map, const int *flags, int *any,
                               void *pack_base, cudaStream_t s);
 // After an unscaled pack: reduces the partial maxima into sA / tB and sets
 // flags[g] (and *any) for operands out of range; flags and *any zeroed by
@@ -255,6 +274,16 @@ cudaError_t launch_tc(TcKind kind, const SplitProb *d_probs, int nprobs,
                       void *pack_base, int64_t pack_rows, const TcConfig &cfg,
                       int *d_err, cudaStream_t s, const int *order = nullptr,
                       int uniform_only = 0, const void *c_maps = nullptr);
+// The same for kTcSplitF16x3 tables (tc_half.cu; bn = 128).  with_d: the product
+// (host copy) of a table of one whose epilogue adds beta D, else nullptr.
+cudaError_t launch_tc_half(const SplitProb *d_probs, int nprobs, int total_units,
+                           const int *unit_map, const int *flags, void *pack_base,
+                           int64_t pack_rows, int grid, int *d_err, cudaStream_t s,
+                           const int *order, const SplitProb *with_d);
+// Tensor map over the pack region viewed as rows of 128 bytes, boxes of bkb
+// (64 or 128) bytes x box_rows rows with the matching swizzle, into `map` (128
+// bytes, 64-byte aligned).
+cudaError_t encode_pack_map(void *map, void *base, int64_t rows, int bkb, int box_rows = 128);
 // Tensor map over C for the tensor-core epilogue's tiled stores (128 bytes
 // written to `map`); usable where tc_c_map_ok holds.
 bool tc_c_map_ok(const float *C, int64_t n, int64_t p);

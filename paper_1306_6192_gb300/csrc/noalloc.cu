@@ -36,6 +36,7 @@ namespace {
 constexpr size_t kNoAllocBytes = (size_t)64 << 20;
 constexpr size_t kFlagOff = 0;      // int timeout flag
 constexpr size_t kScaleFlagOff = 64;  // int per-operand scale flags
+constexpr size_t kHalfOff = 96;     // state words of the fp16 kind (kHalfWords)
 constexpr size_t kTableOff = 256;   // one SplitProb
 constexpr size_t kScalesOff = 512;  // uint32 per row of A and column of B
 static_assert(sizeof(SplitProb) <= kScalesOff - kTableOff, "table slot");
@@ -129,6 +130,7 @@ mm_status mm_gemm_split_static(int64_t n, int64_t m, int64_t p, const float *A, 
   sp.tB = sp.sA + n;
   sp.pA = reinterpret_cast<uint32_t *>(base + part_off);
   sp.pB = sp.pA + (int64_t)sp.kt * n;
+  if (kind == kTcSplitF16x3) sp.hx = reinterpret_cast<int32_t *>(base + kHalfOff);
   sp.unit_start = 0;  // no tail split: split_s = 0 from the memset
   sp.pack_start = 0;
   const int64_t tiles = (int64_t)sp.mt * sp.nt;
@@ -138,7 +140,7 @@ mm_status mm_gemm_split_static(int64_t n, int64_t m, int64_t p, const float *A, 
   // The array keeps the previous call's contents: the timeout and scale flags
   // must start at zero; the maxima and every pack row the kernels read are
   // rewritten (zero padding included) by the pack and verify kernels.
-  cudaError_t e = cudaMemsetAsync(d_flag, 0, 128, s);  // timeout flag and scale flags
+  cudaError_t e = cudaMemsetAsync(d_flag, 0, 128, s);  // timeout, scale and state words
   if (e == cudaSuccess) e = cudaMemsetAsync(sp.sA, 0, (size_t)(n + p) * 4, s);
   if (e == cudaSuccess)
     e = cudaMemcpyAsync(d_tab, &sp, sizeof(sp), cudaMemcpyHostToDevice, s);
@@ -146,7 +148,7 @@ mm_status mm_gemm_split_static(int64_t n, int64_t m, int64_t p, const float *A, 
   // same passes as mm_gemm's split path: unscaled pack with the maxima,
   // verification, re-pack of operands out of range
   if (e == cudaSuccess)
-    e = launch_split_pack(kind, kPackUnscaled, d_tab, 1, (int)packs, nullptr, nullptr, nullptr,
+    e = launch_split_pack(kind, kPackUnscaled, d_tab, 1, (int)packs, nullptr, nullptr, d_sflag + 1,
                           pack, s);
   // d_sflag[0]: the operands' scale flags; d_sflag[1]: set when any is flagged
   if (e == cudaSuccess)
@@ -160,7 +162,10 @@ mm_status mm_gemm_split_static(int64_t n, int64_t m, int64_t p, const float *A, 
     const int grid = ch.grid > 0 ? ch.grid : sms;
     TcConfig cfg = kind == kTcSplitBf16x3 ? TcConfig{2 * ch.bk, ch.stages, grid, ch.bn}
                                           : TcConfig{64, 3, grid, ch.bn};
-    e = launch_tc(kind, d_tab, 1, (int)tiles, nullptr, d_sflag, pack, rows, cfg, d_flag, s);
+    e = kind == kTcSplitF16x3
+            ? launch_tc_half(d_tab, 1, (int)tiles, nullptr, d_sflag, pack, rows,
+                             tc_launch_grid(cfg, tiles), d_flag, s, nullptr, nullptr)
+            : launch_tc(kind, d_tab, 1, (int)tiles, nullptr, d_sflag, pack, rows, cfg, d_flag, s);
   }
   if (e != cudaSuccess) {
     cudaGetLastError();

@@ -57,6 +57,7 @@
 #include <vector>
 
 #include "tc_ptx.cuh"
+#include "tc_units.cuh"
 
 namespace mm {
 namespace {
@@ -64,7 +65,6 @@ namespace {
 constexpr int kThreads = 192;
 constexpr uint32_t kTmemCols = 512;         // all of TMEM: the accumulators
 constexpr int kBoxRows = 128;               // TMA box height (rows of the pack)
-constexpr int kMaxSplit = 4;                // most K parts of a tail-split tile
 constexpr uint64_t kWaitLimitNs = 4000000000ull;
 constexpr uint64_t kDrainLimitNs = 200000000ull;
 
@@ -96,32 +96,6 @@ __device__ __forceinline__ int kind_exponent(uint32_t max_bits) {
   return (f > 0.0f && f <= 3.402823466e38f) ? e - 7 : 0;
 }
 
-// Work unit u of a table: problem g, output tile (mt, nt) = local tile t of
-// the problem in raster order (bands of group_m row tiles), and part h of a
-// tile split along K (h = -1: the whole tile).
-struct UnitCoord {
-  int g, mt, nt, t, h;
-};
-
-__device__ __forceinline__ UnitCoord decode_unit(const SplitProb *__restrict__ probs, int nprobs,
-                                                 const int *__restrict__ map, int u) {
-  const int g =
-      find_problem(probs, nprobs, map, u, [](const SplitProb &q) { return q.unit_start; });
-  const SplitProb &pr = probs[g];
-  int t = u - pr.unit_start, h = -1;
-  if (pr.split_s > 1 && t >= pr.split_from) {
-    const int v = t - pr.split_from;
-    t = pr.split_from + v / pr.split_s;
-    h = v % pr.split_s;
-  }
-  const int gm = pr.group_m;
-  const int band = gm * pr.nt;
-  const int first = (t / band) * gm;
-  const int rows = min(pr.mt - first, gm);
-  const int in = t % band;
-  return UnitCoord{g, first + in % rows, in / rows, t, h};
-}
-
 // FP8 tables with per-block factors: tile (mt, nt) of 128 x 256 keeps one
 // exponent per row and column along K when its row tile and both of its
 // 128-column halves are flagged (pr.cnt: mt row-tile flags, then the flags of
@@ -131,22 +105,6 @@ __device__ __forceinline__ bool skip_unit(const SplitProb &pr, int uniform_only,
   if (!uniform_only) return false;
   const int *f = pr.cnt;
   return !(f[mt] != 0 && f[pr.mt + 2 * nt] != 0 && f[pr.mt + 2 * nt + 1] != 0);
-}
-
-// Pipeline stages [k0, k1) of a unit: all kiters of a whole tile; for part h
-// the stages of pack rows [h*kt/S, (h+1)*kt/S), so the split points do not
-// depend on the stage depth BKB.
-template <int BKB>
-__device__ __forceinline__ void unit_krange(const SplitProb &pr, int h, int kiters, int &k0,
-                                            int &k1) {
-  if (h < 0) {
-    k0 = 0;
-    k1 = kiters;
-    return;
-  }
-  constexpr int kStagesPerRow = kPackRowBytes / BKB;
-  k0 = (int)((int64_t)h * pr.kt / pr.split_s) * kStagesPerRow;
-  k1 = min((int)((int64_t)(h + 1) * pr.kt / pr.split_s) * kStagesPerRow, kiters);
 }
 
 __device__ __forceinline__ void epilogue_sync() {
@@ -610,23 +568,23 @@ PFN_cuTensorMapEncodeTiled_v12000 get_encode_fn() {
   return fn;
 }
 
+}  // namespace
+
 // 2-D map over the pack region viewed as rows of 128 bytes; a box is BKB
-// bytes of 128 consecutive rows.
-cudaError_t encode_pack_map(CUtensorMap *map, void *base, int64_t rows, int bkb) {
+// bytes of box_rows consecutive rows.
+cudaError_t encode_pack_map(void *map, void *base, int64_t rows, int bkb, int box_rows) {
   auto enc = get_encode_fn();
   if (!enc) return cudaErrorNotSupported;
   cuuint64_t dims[2] = {(cuuint64_t)kPackRowBytes, (cuuint64_t)rows};
   cuuint64_t strides[1] = {(cuuint64_t)kPackRowBytes};
-  cuuint32_t box[2] = {(cuuint32_t)bkb, (cuuint32_t)kBoxRows};
+  cuuint32_t box[2] = {(cuuint32_t)bkb, (cuuint32_t)box_rows};
   cuuint32_t estr[2] = {1, 1};
-  CUresult r = enc(map, CU_TENSOR_MAP_DATA_TYPE_UINT8, 2, base, dims, strides, box, estr,
+  CUresult r = enc(static_cast<CUtensorMap *>(map), CU_TENSOR_MAP_DATA_TYPE_UINT8, 2, base, dims, strides, box, estr,
                    CU_TENSOR_MAP_INTERLEAVE_NONE,
                    bkb == 128 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B,
                    CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
 }
-
-}  // namespace
 
 // 2-D map over C (n rows of p FP32, row-major) for the epilogue's tiled
 // stores: boxes of 32 x 32 with a 128-byte swizzle.  Needs a 16-byte aligned

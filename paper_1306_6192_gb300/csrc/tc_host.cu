@@ -11,7 +11,7 @@ namespace mm {
 
 TcKind split_kind_for(int64_t m) {
   return 3.1 * std::ldexp(1.0, -16) <= 1e-6 * std::sqrt((double)m) ? kTcSplitBf16x3
-                                                                    : kTcSplitBf16x6;
+                                                                    : kTcSplitF16x3;
 }
 
 namespace {
@@ -26,7 +26,7 @@ struct Group {
 };
 
 double kind_products(TcKind k) {
-  return k == kTcSplitBf16x3 ? 3.0 : (k == kTcSplitBf16x6 ? 6.0 : 0.5);
+  return k == kTcSplitBf16x6 ? 6.0 : (k == kTcE4m3 ? 0.5 : 3.0);
 }
 
 // Tail split of one product from its own shape and tile choice; fills
@@ -43,8 +43,8 @@ TcTail plan_tail(SplitProb &sp, TcKind kind, const TcChoice &ch) {
 
 mm_status run_tc_groups(Scratch &ws, const mm_problem *probs, int count, cudaStream_t s,
                         const TcChoice *force, bool six, const Epi *epi) {
-  Group groups[2] = {{kTcSplitBf16x3}, {kTcSplitBf16x6}};
-  int64_t rows = 0, scal = 0, part = 0;
+  Group groups[2] = {{kTcSplitBf16x3}, {six ? kTcSplitBf16x6 : kTcSplitF16x3}};
+  int64_t rows = 0, scal = 0, part = 0, half = 0;
   size_t tail_parts = 0, tail_cnts = 0;  // partial tiles and counters of tail splits
   for (int g = 0; g < count; g++) {
     const mm_problem &q = probs[g];
@@ -90,6 +90,8 @@ mm_status run_tc_groups(Scratch &ws, const mm_problem *probs, int count, cudaStr
     part += (int64_t)sp.kt * q.n;
     sp.pB = reinterpret_cast<uint32_t *>((uintptr_t)part);
     part += (int64_t)sp.kt * q.p;
+    // state words of the fp16 kind (offset + 1, fixed below)
+    if (kind == kTcSplitF16x3) sp.hx = reinterpret_cast<int32_t *>((uintptr_t)(++half));
     sp.ver_start = (int32_t)G.vers;
     G.vers += verify_items(q.n, q.p);
     G.max_kt = std::max(G.max_kt, sp.kt);
@@ -98,7 +100,7 @@ mm_status run_tc_groups(Scratch &ws, const mm_problem *probs, int count, cudaStr
       sp.part = reinterpret_cast<float *>((uintptr_t)tail_parts);
       sp.cnt = reinterpret_cast<int *>((uintptr_t)tail_cnts);
       tail_parts += tc_tail_part_bytes(tail, (int64_t)sp.mt * sp.nt, sp.bn);
-      tail_cnts += (size_t)((int64_t)sp.mt * sp.nt - tail.split_from);
+      tail_cnts += (size_t)((int64_t)sp.mt * sp.nt - tail.split_from) * (sp.hx ? kHalfSplitCnt : 1);
     }
     sp.unit_start = (int32_t)G.units;
     G.units += split_units(sp);
@@ -116,13 +118,14 @@ mm_status run_tc_groups(Scratch &ws, const mm_problem *probs, int count, cudaStr
   if (ntab == 0) return MM_OK;
   if (rows > 0x7fffffffLL) return MM_EINVAL;
   // Layout: packs | the words that start at zero (scale words, per-problem
-  // scale flags and one "any flagged" word per group, tail-split counters: one
-  // memset clears them) | partial maxima | table | item maps | partial tiles
+  // scale flags and one "any flagged" word per group, tail-split counters,
+  // fp16 state words: one memset clears them) | partial maxima | table | item maps | partial tiles
   const size_t pack_bytes = (size_t)rows * kPackRowBytes;
   const size_t scal_off = (pack_bytes + 255) & ~(size_t)255;
   const size_t flag_off = scal_off + (size_t)scal * 4;
   const size_t tcnt_off = flag_off + (ntab + 3) * sizeof(int);
-  const size_t zero_end = tcnt_off + tail_cnts * sizeof(int);
+  const size_t half_off = (tcnt_off + tail_cnts * sizeof(int) + 15) & ~(size_t)15;
+  const size_t zero_end = half_off + (size_t)half * kHalfWords * sizeof(int);
   const size_t part_off = (zero_end + 255) & ~(size_t)255;
   const size_t tab_off = (part_off + (size_t)part * 4 + 255) & ~(size_t)255;
   // item -> problem maps (work units, pack tiles and verify items) of each
@@ -160,6 +163,8 @@ mm_status run_tc_groups(Scratch &ws, const mm_problem *probs, int count, cudaStr
       sp.tB = reinterpret_cast<uint32_t *>(base + scal_off) + (uintptr_t)sp.tB;
       sp.pA = reinterpret_cast<uint32_t *>(base + part_off) + (uintptr_t)sp.pA;
       sp.pB = reinterpret_cast<uint32_t *>(base + part_off) + (uintptr_t)sp.pB;
+      if (sp.hx)
+        sp.hx = reinterpret_cast<int32_t *>(base + half_off) + ((uintptr_t)sp.hx - 1) * kHalfWords;
       if (sp.split_s > 1) {
         sp.part = reinterpret_cast<float *>(base + tpart_off + (uintptr_t)sp.part);
         sp.cnt = reinterpret_cast<int *>(base + tcnt_off) + (uintptr_t)sp.cnt;
@@ -174,6 +179,7 @@ mm_status run_tc_groups(Scratch &ws, const mm_problem *probs, int count, cudaStr
     std::vector<uint8_t> blob(cmap_rel + cmap_bytes, 0);
     for (size_t k = 0; cmap_bytes && k < ntab; k++) {
       SplitProb &sp = all[k];
+      if (sp.hx) continue;  // tc_half.cu stores whole sectors from registers
       // the epilogue C = alpha (A.B) + beta D loads D in 16-byte vectors
       // beside the tiled stores (a D off that alignment: plain stores)
       const bool d_ok = sp.epi.on != 2 || (reinterpret_cast<uintptr_t>(sp.epi.D) & 15u) == 0;
@@ -218,16 +224,21 @@ mm_status run_tc_groups(Scratch &ws, const mm_problem *probs, int count, cudaStr
       e = launch_split_maps(dt, np, tile_map, pack_map, ver_map, s);
       if (e != cudaSuccess) return note_cuda(e);
     }
+
     // one unscaled pass that also reduces the maxima, then the operands out
     // of range are re-packed with their scales
-    e = launch_split_pack(G.kind, kPackUnscaled, dt, np, (int)G.packs, pack_map, nullptr, nullptr,
+    e = launch_split_pack(G.kind, kPackUnscaled, dt, np, (int)G.packs, pack_map, nullptr, any,
                           base, s);
     if (e == cudaSuccess) e = launch_split_verify(dt, np, G.vers, ver_map, flags, any, G.max_kt, s);
     if (e == cudaSuccess)
       e = launch_split_pack(G.kind, kPackFix, dt, np, (int)G.packs, pack_map, flags, any, base, s);
     if (e == cudaSuccess)
-      e = launch_tc(G.kind, dt, np, (int)G.units, tile_map, flags, base, rows, G.cfg, g_ctx.d_err,
-                    s, order, 0, d_cmaps);
+      e = G.kind == kTcSplitF16x3
+              ? launch_tc_half(dt, np, (int)G.units, tile_map, flags, base, rows,
+                               tc_launch_grid(G.cfg, G.units), g_ctx.d_err, s, order,
+                               G.tab[0].epi.on == 2 ? &G.tab[0] : nullptr)
+              : launch_tc(G.kind, dt, np, (int)G.units, tile_map, flags, base, rows, G.cfg, g_ctx.d_err,
+                          s, order, 0, d_cmaps);
     if (e != cudaSuccess) return note_cuda(e);
   }
   return MM_OK;
@@ -239,7 +250,9 @@ mm_status run_split_chunked(Scratch &ws, int64_t n, int64_t m, int64_t p, const 
                             const float *B, float *C, int chunks, const int64_t *row0,
                             cudaStream_t s, cudaEvent_t *in_ready, cudaEvent_t *out_ready) {
   if (n == 0 || p == 0) return MM_OK;
-  const TcKind kind = split_kind_for(m);
+  // the slabs of A share one pack of B, so the choice between fp16 and bf16
+  // parts cannot wait for the last slab to arrive: three bf16 parts
+  const TcKind kind = split_kind_for(m) == kTcSplitBf16x3 ? kTcSplitBf16x3 : kTcSplitBf16x6;
   const int parts = pack_parts(kind);
   TcChoice ch = tune_choose(n, m, p);
   ch.bn = tc_bn(kind, ch.bn);
@@ -420,7 +433,7 @@ FusedPlan fused_plan(int64_t n, int64_t m, int64_t p, TcKind kind) {
   // products that fill at least half of the SMs with whole tiles keep the
   // packed path (their operands are converted once, not once per tile)
   if (2 * tiles > sm_count()) return best;
-  const bool six = kind == kTcSplitBf16x6;
+  const bool six = kind != kTcSplitBf16x3;
   // cost in units of one K block of one CTA (its conversion dominates): the
   // blocks of the longest slice, the cluster's exchange through distributed
   // shared memory, and the clusters' meeting in global memory, whose last
@@ -483,7 +496,7 @@ mm_status run_fused(Scratch &ws, int64_t n, int64_t m, int64_t p, const float *A
     fp.cnt = static_cast<int *>(ws.ptr);
     fp.slots = reinterpret_cast<float *>(static_cast<uint8_t *>(ws.ptr) + cnt_bytes);
   }
-  e = launch_fused(kind == kTcSplitBf16x6, fp, plan.cs, g_ctx.d_err, s);
+  e = launch_fused(kind != kTcSplitBf16x3, fp, plan.cs, g_ctx.d_err, s);
   return note_cuda(e);
 }
 
