@@ -69,8 +69,47 @@ cudaError_t Scratch::reserve(size_t need, cudaStream_t s) {
   return cudaSuccess;
 }
 
+cudaError_t Scratch::take_words(size_t counters, cudaStream_t s, int **state, int **clear) {
+  cudaError_t e = cudaSuccess;
+  if (!words) {
+    e = cudaMalloc(&words, kWords * sizeof(int));
+    if (e != cudaSuccess) {
+      cudaGetLastError();
+      words = nullptr;
+      return cudaErrorMemoryAllocation;
+    }
+    words_epoch = 0;
+  }
+  if (3 * kStateWords + counters > kWords) return cudaErrorInvalidValue;
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  e = cudaStreamIsCapturing(s, &cap);
+  if (e != cudaSuccess) return e;
+  const bool captured = cap != cudaStreamCaptureStatusNone;
+  // a launch or a wait that failed may have left words set
+  if (words_epoch != g_ctx.err_epoch) {
+    e = cudaMemsetAsync(words, 0, kWords * sizeof(int), s);
+    if (e != cudaSuccess) return e;
+    if (!captured) words_epoch = g_ctx.err_epoch;
+  }
+  if (captured) {
+    // a replay does not alternate with other calls: a set of its own, cleared
+    // ahead of its kernels
+    *state = words + 2 * kStateWords;
+    *clear = nullptr;
+    return cudaMemsetAsync(*state, 0, kStateWords * sizeof(int), s);
+  }
+  *state = words + words_turn * kStateWords;
+  words_turn ^= 1;
+  *clear = words + words_turn * kStateWords;
+  return cudaSuccess;
+}
+
 void Scratch::release() {
   if (ptr) cudaFree(ptr);
+  if (words) cudaFree(words);
+  words = nullptr;
+  words_turn = 0;
+  words_epoch = 0;
   ptr = nullptr;
   bytes = 0;
   stage.release();
@@ -292,13 +331,20 @@ mm_status enqueue_gemm(int64_t n, int64_t m, int64_t p, const void *A, const voi
       // output tiles run as one fused split-K launch
       const TcKind kind = split_kind_of(md, m);
       const FusedPlan fpl = fused_plan(n, m, p, kind);
-      if (fpl.S > 0 && fused_operands_ok(static_cast<const float *>(A),
-                                         static_cast<const float *>(B), m, p)) {
+      const bool fused = fpl.S > 0 && fused_operands_ok(static_cast<const float *>(A),
+                                                        static_cast<const float *>(B), m, p);
+      // with m < 2237 and more than three K blocks a slice the packed fp16 form is
+      // faster: the fused kernel converts every operand for each of its tiles
+      // (GB300, fused against packed: 512^3 at one block 17 / 19 us, 300 x 2236 x
+      // 300 at three 26 / 29, 1024 x 1024 x 512 at four 26 / 24.5, 1024^3 at eight
+      // 44.5 / 25.1)
+      if (fused && (kind != kTcSplitF16x3 || ceil_div(ceil_div(m, 64), fpl.S) <= 3)) {
         return run_fused(g_ctx.fused_ws, n, m, p, static_cast<const float *>(A),
                          static_cast<const float *>(B), static_cast<float *>(C), kind, fpl, s, epi);
       }
       mm_problem q{n, m, p, A, B, C};
-      return run_split(g_ctx.split_ws, &q, 1, s, nullptr, md == MM_MODE_SPLIT_BF16X6, epi);
+      return run_split(g_ctx.split_ws, &q, 1, s, nullptr, md == MM_MODE_SPLIT_BF16X6, epi,
+                       fused ? kHalfShortChunk : kHalfChunk);
     }
     case MM_MODE_FP8: {
       // the e4m3 tiles' MMAs take about as long as their stores, so the
@@ -324,7 +370,8 @@ mm_status check_device_flag(cudaStream_t s) {
   if (e != cudaSuccess) return note_cuda(e);
   if (flag != 0) {
     cudaMemset(g_ctx.d_err, 0, sizeof(int));
-    g_ctx.fused_zero_ptr = nullptr;  // an aborted fused launch may leave counters set
+    g_ctx.fused_zero_ptr = nullptr;  // an aborted launch may leave counters and words set
+    g_ctx.err_epoch++;
     return MM_ETIMEOUT;
   }
   return MM_OK;

@@ -26,6 +26,19 @@ struct Scratch {
   void *ptr = nullptr;
   size_t bytes = 0;
   HostStage stage;  // host side of the tables written into this scratch
+  // Words that are zero between calls (calls on one scratch are ordered on one
+  // stream): two sets of kStateWords, used in turn, of which each call clears
+  // the other's in its last kernel, one for captured calls, and the tail
+  // split's counters, which its last parts reset.  Valid while words_epoch is the library's error epoch.
+  int *words = nullptr;
+  int words_turn = 0;
+  uint64_t words_epoch = 0;
+  static constexpr size_t kWords = 8 * 1024;
+  // The state words of the next call on one product (zero on the device when
+  // its first kernel runs) and those its last kernel clears; `counters` tail
+  // counters must be zero, too.
+  cudaError_t take_words(size_t counters, cudaStream_t s, int **state, int **clear);
+  int *counters() const { return words + 3 * kStateWords; }
   // Makes room for `need` bytes; an existing buffer is freed after `s` has
   // drained (its contents are not kept).
   cudaError_t reserve(size_t need, cudaStream_t s);
@@ -65,6 +78,7 @@ struct Ctx {
   Scratch epi_ws;        // the product of an in-place epilogue run as a second pass
   void *fused_zero_ptr = nullptr;  // fused_ws buffer whose leading counters are zero
   size_t fused_zeroed = 0;         //   and how many bytes of them
+  uint64_t err_epoch = 1;  // counts the device-side waits that ran out
   int ozaki_slices = kOzakiDefaultSlices;  // digit slices S of MM_MODE_OZAKI
   int ozaki_gate = 1;                      // accuracy gate of MM_MODE_OZAKI on
   // host-operand pipeline of mm_gemm: copy streams and per-chunk events
@@ -121,9 +135,14 @@ inline int tc_bn(TcKind kind, int bn) {
 // problem takes the kind split_kind_for(m).  `force` overrides the tuned tile
 // choice (autotuner and tests).
 // `six` selects the three-part kind (six products) for every problem.
-// `epi` (null: C = A.B) is the epilogue of a table of one product.
+// `epi` (null: C = A.B) is the epilogue of a table of one product.  `chunk`: K
+// blocks summed in one accumulator of the fp16 form (kHalfChunk; a shorter one
+// costs 3-5% and halves the accumulation error: 512 K 6.4e-7 of the result's
+// norm at 1024^3, 256 K 3.5e-7, the fused kernel's 64 K of six products 4.0e-7).
+constexpr int kHalfChunk = 8, kHalfShortChunk = 4;
 mm_status run_split(Scratch &ws, const mm_problem *probs, int count, cudaStream_t s,
-                    const TcChoice *force, bool six = false, const Epi *epi = nullptr);
+                    const TcChoice *force, bool six = false, const Epi *epi = nullptr,
+                    int chunk = kHalfChunk);
 // Split path for one product whose rows of A (and of C) are processed in
 // `chunks` slabs: slab c waits for event in_ready[c + 1] (B: in_ready[0])
 // before its prep and records out_ready[c] when its part of C is written.

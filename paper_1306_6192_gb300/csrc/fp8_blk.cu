@@ -718,8 +718,8 @@ mm_status fp8_blocks_launch(Scratch &ws, std::vector<SplitProb> &blk, std::vecto
     blk_map = reinterpret_cast<int *>(base + map_off);
     tc_map = blk_map + blk_units;
     pack_map = tc_map + tc_units;
-    e = launch_split_maps(d_blk, np, blk_map, nullptr, nullptr, s);
-    if (e == cudaSuccess) e = launch_split_maps(d_tc, np, tc_map, pack_map, nullptr, s);
+    e = launch_split_maps(device_table(d_blk, np), blk_map, nullptr, nullptr, s);
+    if (e == cudaSuccess) e = launch_split_maps(device_table(d_tc, np), tc_map, pack_map, nullptr, s);
     if (e != cudaSuccess) return note_cuda(e);
   }
   {
@@ -733,7 +733,7 @@ mm_status fp8_blocks_launch(Scratch &ws, std::vector<SplitProb> &blk, std::vecto
   // the uniform 128 x 256 tiles: one factor per row and column
   TcConfig cfg{128, 4, 0};
   cfg.max_bn = kPackBN;
-  e = launch_tc(kTcE4m3, d_tc, np, (int)tc_units, tc_map, nullptr, ws.ptr, rows, cfg, g_ctx.d_err,
+  e = launch_tc(kTcE4m3, device_table(d_tc, np), (int)tc_units, tc_map, nullptr, ws.ptr, rows, cfg, g_ctx.d_err,
                 s, nullptr, 1, d_cmaps);
   if (e != cudaSuccess) return note_cuda(e);
   // the other tiles, K block by K block

@@ -128,6 +128,8 @@ struct SplitProb {
   int32_t c_tma;
   // kTcSplitF16x3: the product's state words (HalfState) on the device
   int32_t *hx;
+  // K blocks that it sums in one accumulator (a power of two)
+  int32_t chunk;
   // C = alpha (A.B) + beta D (plain stores only; off: C = A.B)
   EpiF epi;
 };
@@ -148,6 +150,21 @@ constexpr int kHalfSplitCnt = 8;
 __host__ __device__ inline int64_t split_units(const SplitProb &sp) {
   const int64_t tiles = (int64_t)sp.mt * sp.nt;
   return sp.split_s > 1 ? sp.split_from + (tiles - sp.split_from) * sp.split_s : tiles;
+}
+
+// A table of products as the kernels take it: an array on the device, or (dev
+// null, n = 1) one product carried in the launch itself, which needs no copy
+// to the device ahead of it.
+struct ProbTable {
+  const SplitProb *dev;
+  int n;
+  SplitProb one;
+};
+inline ProbTable device_table(const SplitProb *d, int n) {
+  ProbTable t{};
+  t.dev = d;
+  t.n = n;
+  return t;
 }
 
 // One product of the fused split-K path (tc_fused.cu): output tiles of
@@ -218,18 +235,21 @@ cudaError_t launch_simt_splitk_f64(int64_t n, int64_t m, int64_t p, const double
 // `map` arguments: item -> problem index arrays written by
 // launch_split_maps for tables of several problems, or nullptr.
 // Also writes the state words of kTcSplitF16x3 products (SplitProb::hx).
-cudaError_t launch_split_maps(const SplitProb *d_probs, int nprobs, int *unit_map,
+cudaError_t launch_split_maps(const ProbTable &tab, int *unit_map,
                               int *pack_map, int *ver_map, cudaStream_t s);
 // Verify items of a product: 32 rows/columns each.
 __host__ __device__ inline int64_t verify_items(int64_t n, int64_t p) { return (n + p + 31) / 32; }
 // Pack modes (split kinds) and the per-problem flags they use.
 constexpr int kPackUnscaled = 1, kPackFix = 2;
 constexpr int kFlagScaleA = 1, kFlagScaleB = 2;
+// Words of a call on one product that start at zero: its flags, its "any
+// flagged" word, and from kStateHalf on its kTcSplitF16x3 state words.
+constexpr int kStateFlags = 0, kStateAny = 1, kStateHalf = 4, kStateWords = 16;
 // kPackUnscaled: one block per pack tile.  kPackFix: a persistent grid that
 // returns at once unless *any is set, then re-packs the tiles of flagged
 // operands (flags[g]).
-cudaError_t launch_split_pack(TcKind kind, int mode, const SplitProb *d_probs, int nprobs,
-                              int total_tiles, const int *map, const int *flags, int *any,
+cudaError_t launch_split_pack(TcKind kind, int mode, const ProbTable &tab, int total_tiles,
+                              const int *map, const int *flags, int *any,
                               void *pack_base, cudaStream_t s);
 // After an unscaled pack: reduces the partial maxima into sA / tB and sets
 // flags[g] (and *any) for operands out of range; flags and *any zeroed by
@@ -238,7 +258,7 @@ cudaError_t launch_split_pack(TcKind kind, int mode, const SplitProb *d_probs, i
 // largest kt of the table.  write_cols = false leaves tB as it is (a later
 // slab sharing B's words, which another stream may be reading) but still
 // flags B.
-cudaError_t launch_split_verify(const SplitProb *d_probs, int nprobs, int64_t total_items,
+cudaError_t launch_split_verify(const ProbTable &tab, int64_t total_items,
                                 const int *map, int *flags, int *any, int max_kt, cudaStream_t s,
                                 bool write_cols = true);
 // Tensor-core mainloop + epilogue over all work units of all problems.
@@ -269,17 +289,18 @@ size_t tc_tail_part_bytes(const TcTail &t, int64_t tiles, int bn);
 // device), or nullptr for units c, c + grid, c + 2 grid, ... on CTA c.
 // uniform_only (FP8 with per-block factors): only the tiles whose rows and
 // columns keep one exponent along K (flags in each problem's cnt) run.
-cudaError_t launch_tc(TcKind kind, const SplitProb *d_probs, int nprobs,
-                      int total_units, const int *unit_map, const int *flags,
+// clear: device words (kStateWords of them) that the launch sets to zero, or
+// nullptr.
+cudaError_t launch_tc(TcKind kind, const ProbTable &tab, int total_units, const int *unit_map,
+                      const int *flags,
                       void *pack_base, int64_t pack_rows, const TcConfig &cfg,
                       int *d_err, cudaStream_t s, const int *order = nullptr,
-                      int uniform_only = 0, const void *c_maps = nullptr);
-// The same for kTcSplitF16x3 tables (tc_half.cu; bn = 128).  with_d: the product
-// (host copy) of a table of one whose epilogue adds beta D, else nullptr.
-cudaError_t launch_tc_half(const SplitProb *d_probs, int nprobs, int total_units,
+                      int uniform_only = 0, const void *c_maps = nullptr, int *clear = nullptr);
+// The same for kTcSplitF16x3 tables (tc_half.cu; bn = 128).
+cudaError_t launch_tc_half(const ProbTable &tab, int total_units,
                            const int *unit_map, const int *flags, void *pack_base,
                            int64_t pack_rows, int grid, int *d_err, cudaStream_t s,
-                           const int *order, const SplitProb *with_d);
+                           const int *order, int *clear);
 // Tensor map over the pack region viewed as rows of 128 bytes, boxes of bkb
 // (64 or 128) bytes x box_rows rows with the matching swizzle, into `map` (128
 // bytes, 64-byte aligned).
@@ -332,6 +353,52 @@ struct TraceScope {
 };
 
 int sm_count();
+
+#ifdef __CUDACC__
+// Launch as a programmatic dependent of the stream's previous kernel: the
+// blocks may become resident while that kernel finishes.  The kernel calls
+// pdl_wait() in every block before it touches global memory that earlier work
+// on the stream writes or reads.  (The four kernels of a packed product with
+// their table in the launch: 47.7 us -> 41.6 us for 1501 x 1999 x 1277.)
+// Grids of many waves go without (dependent = false): the two-part pack of
+// 8192^3, 32,768 blocks, made the call 1% slower as a dependent (2025 us against
+// 2003), each block passing through the wait.
+template <typename... KArgs, typename... Args>
+cudaError_t launch_pdl_if(bool dependent, void (*kernel)(KArgs...), unsigned grid, unsigned block,
+                          size_t smem, cudaStream_t s, Args... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(grid, 1, 1);
+  cfg.blockDim = dim3(block, 1, 1);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = dependent ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, kernel, args...);
+}
+template <typename... KArgs, typename... Args>
+cudaError_t launch_pdl(void (*kernel)(KArgs...), unsigned grid, unsigned block, size_t smem,
+                       cudaStream_t s, Args... args) {
+  return launch_pdl_if(true, kernel, grid, block, smem, s, args...);
+}
+// The table's products; one carried in the launch is copied into the block's
+// shared memory (by all its threads; a barrier must follow), where every role
+// reads it tile after tile.
+__device__ __forceinline__ const SplitProb *table_products(const ProbTable &tab, SplitProb *shared_one) {
+  if (tab.dev) return tab.dev;
+  static_assert(sizeof(SplitProb) % 4 == 0, "copied in words");
+  for (unsigned i = threadIdx.x; i < sizeof(SplitProb) / 4; i += blockDim.x)
+    reinterpret_cast<uint32_t *>(shared_one)[i] = reinterpret_cast<const uint32_t *>(&tab.one)[i];
+  return shared_one;
+}
+// Waits for the stream's earlier work, then lets the next kernel's blocks in.
+__device__ __forceinline__ void pdl_wait() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+#endif
 
 // Status from a CUDA error code.
 mm_status from_cuda(cudaError_t e);

@@ -37,9 +37,7 @@ constexpr size_t kNoAllocBytes = (size_t)64 << 20;
 constexpr size_t kFlagOff = 0;      // int timeout flag
 constexpr size_t kScaleFlagOff = 64;  // int per-operand scale flags
 constexpr size_t kHalfOff = 96;     // state words of the fp16 kind (kHalfWords)
-constexpr size_t kTableOff = 256;   // one SplitProb
 constexpr size_t kScalesOff = 512;  // uint32 per row of A and column of B
-static_assert(sizeof(SplitProb) <= kScalesOff - kTableOff, "table slot");
 constexpr int kMaxDevices = 64;
 
 static __device__ __align__(256) uint8_t g_noalloc_scratch[kNoAllocBytes];
@@ -130,32 +128,31 @@ mm_status mm_gemm_split_static(int64_t n, int64_t m, int64_t p, const float *A, 
   sp.tB = sp.sA + n;
   sp.pA = reinterpret_cast<uint32_t *>(base + part_off);
   sp.pB = sp.pA + (int64_t)sp.kt * n;
+  sp.chunk = kHalfChunk;
   if (kind == kTcSplitF16x3) sp.hx = reinterpret_cast<int32_t *>(base + kHalfOff);
   sp.unit_start = 0;  // no tail split: split_s = 0 from the memset
   sp.pack_start = 0;
   const int64_t tiles = (int64_t)sp.mt * sp.nt;
   const int64_t packs = (int64_t)sp.mt * sp.kt + (int64_t)sp.nt * sp.kt;
-  SplitProb *d_tab = reinterpret_cast<SplitProb *>(base + kTableOff);
+  ProbTable tab{nullptr, 1, sp};
   int *d_flag = reinterpret_cast<int *>(base + kFlagOff);
   // The array keeps the previous call's contents: the timeout and scale flags
   // must start at zero; the maxima and every pack row the kernels read are
   // rewritten (zero padding included) by the pack and verify kernels.
   cudaError_t e = cudaMemsetAsync(d_flag, 0, 128, s);  // timeout, scale and state words
   if (e == cudaSuccess) e = cudaMemsetAsync(sp.sA, 0, (size_t)(n + p) * 4, s);
-  if (e == cudaSuccess)
-    e = cudaMemcpyAsync(d_tab, &sp, sizeof(sp), cudaMemcpyHostToDevice, s);
   int *d_sflag = reinterpret_cast<int *>(base + kScaleFlagOff);
   // same passes as mm_gemm's split path: unscaled pack with the maxima,
   // verification, re-pack of operands out of range
   if (e == cudaSuccess)
-    e = launch_split_pack(kind, kPackUnscaled, d_tab, 1, (int)packs, nullptr, nullptr, d_sflag + 1,
+    e = launch_split_pack(kind, kPackUnscaled, tab, (int)packs, nullptr, nullptr, d_sflag + 1,
                           pack, s);
   // d_sflag[0]: the operands' scale flags; d_sflag[1]: set when any is flagged
   if (e == cudaSuccess)
-    e = launch_split_verify(d_tab, 1, verify_items(n, p), nullptr, d_sflag, d_sflag + 1, sp.kt,
+    e = launch_split_verify(tab, verify_items(n, p), nullptr, d_sflag, d_sflag + 1, sp.kt,
                             s);
   if (e == cudaSuccess)
-    e = launch_split_pack(kind, kPackFix, d_tab, 1, (int)packs, nullptr, d_sflag, d_sflag + 1,
+    e = launch_split_pack(kind, kPackFix, tab, (int)packs, nullptr, d_sflag, d_sflag + 1,
                           pack, s);
   if (e == cudaSuccess) {
     // the tuned grid (0: one CTA per SM of this device, counted at set-up)
@@ -163,9 +160,9 @@ mm_status mm_gemm_split_static(int64_t n, int64_t m, int64_t p, const float *A, 
     TcConfig cfg = kind == kTcSplitBf16x3 ? TcConfig{2 * ch.bk, ch.stages, grid, ch.bn}
                                           : TcConfig{64, 3, grid, ch.bn};
     e = kind == kTcSplitF16x3
-            ? launch_tc_half(d_tab, 1, (int)tiles, nullptr, d_sflag, pack, rows,
+            ? launch_tc_half(tab, (int)tiles, nullptr, d_sflag, pack, rows,
                              tc_launch_grid(cfg, tiles), d_flag, s, nullptr, nullptr)
-            : launch_tc(kind, d_tab, 1, (int)tiles, nullptr, d_sflag, pack, rows, cfg, d_flag, s);
+            : launch_tc(kind, tab, (int)tiles, nullptr, d_sflag, pack, rows, cfg, d_flag, s);
   }
   if (e != cudaSuccess) {
     cudaGetLastError();

@@ -710,7 +710,7 @@ mm_status run_ozaki(Scratch &ws, int64_t n, int64_t m, int64_t p, const double *
                                                                           tiles);
     if ((e = cudaGetLastError()) != cudaSuccess) return note_cuda(e);
   }
-  e = launch_tc(kTcE4m3, d_tab, nprobs, (int)lay.units, unit_map, nullptr, ws.ptr, lay.rows, cfg,
+  e = launch_tc(kTcE4m3, device_table(d_tab, nprobs), (int)lay.units, unit_map, nullptr, ws.ptr, lay.rows, cfg,
                 g_ctx.d_err, s, d_order);
   if (e != cudaSuccess) return note_cuda(e);
   // the gate reads the level sums only, so it runs before the sum kernel:

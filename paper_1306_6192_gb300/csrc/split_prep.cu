@@ -300,10 +300,13 @@ __device__ __forceinline__ void pack_a_tile(const SplitProb &pr, int local, uint
 // thread keeps several loads in flight.
 template <int PARTS, int MODE>
 __global__ void __launch_bounds__(256, 4)
-split_pack_kernel(const SplitProb *__restrict__ probs, int nprobs, const int *__restrict__ map,
+split_pack_kernel(const __grid_constant__ ProbTable tab, const int *__restrict__ map,
                   const int *__restrict__ flags, const int *__restrict__ any, int total_tiles,
                   uint2 *__restrict__ pack) {
   __shared__ float tile[kPackK][128 + 1];
+  const SplitProb *probs = tab.dev ? tab.dev : &tab.one;
+  const int nprobs = tab.n;
+  pdl_wait();
   if (MODE == kPackFix && *any == 0) return;
   const int tid = threadIdx.x;
   for (int item = blockIdx.x; item < total_tiles; item += gridDim.x) {
@@ -483,13 +486,16 @@ __device__ __forceinline__ bool emit_tile(const PackItem &d, const float4 *t4, i
 }
 
 __global__ void __launch_bounds__(288, 2)
-split_pack_half_kernel(const SplitProb *__restrict__ probs, int nprobs, const int *__restrict__ map,
+split_pack_half_kernel(const __grid_constant__ ProbTable tab, const int *__restrict__ map,
                        int *any, int total_tiles, uint2 *__restrict__ pack) {
   extern __shared__ __align__(16) float4 tiles[];  // kPkStages of 128 x 64 entries
   __shared__ PackItem items[kPkItems];
   __shared__ uint32_t mx_s[8], mn_s[8];
   __shared__ int one[3];  // the state words of a table of one product
+  const SplitProb *probs = tab.dev ? tab.dev : &tab.one;
+  const int nprobs = tab.n;
   const int tid = threadIdx.x;
+  pdl_wait();
   if (map == nullptr && tid < 256) {
     int ea, eb;
     const uint2 ra = sample_range(probs->A, (int64_t)probs->n * probs->m, mx_s, mn_s);
@@ -575,10 +581,13 @@ split_pack_half_kernel(const SplitProb *__restrict__ probs, int nprobs, const in
 
 // The fix pass of such a table (a persistent grid, as split_pack_kernel's).
 __global__ void __launch_bounds__(256, 4)
-split_fix_half_kernel(const SplitProb *__restrict__ probs, int nprobs, const int *__restrict__ map,
+split_fix_half_kernel(const __grid_constant__ ProbTable tab, const int *__restrict__ map,
                       const int *__restrict__ flags, const int *__restrict__ any, int total_tiles,
                       uint2 *__restrict__ pack) {
   __shared__ float tile[kPackK][128 + 1];
+  const SplitProb *probs = tab.dev ? tab.dev : &tab.one;
+  const int nprobs = tab.n;
+  pdl_wait();
   if (*any == 0) return;
   for (int item = blockIdx.x; item < total_tiles; item += gridDim.x) {
     const int g =
@@ -607,10 +616,13 @@ __device__ __forceinline__ bool needs_scale(uint32_t max_bits) {
 // unscaled.
 template <int WPI>
 __global__ void __launch_bounds__(256)
-split_verify_kernel(const SplitProb *__restrict__ probs, int nprobs, const int *__restrict__ map,
+split_verify_kernel(const __grid_constant__ ProbTable tab, const int *__restrict__ map,
                     int total_items, int *__restrict__ flags, int *__restrict__ any,
                     bool write_cols) {
   __shared__ uint32_t part[8][32];
+  const SplitProb *probs = tab.dev ? tab.dev : &tab.one;
+  const int nprobs = tab.n;
+  pdl_wait();
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int sub = warp % WPI;
   const int item = blockIdx.x * (8 / WPI) + warp / WPI;
@@ -662,11 +674,12 @@ split_verify_kernel(const SplitProb *__restrict__ probs, int nprobs, const int *
 // tiles, pack tiles and scale-reduction items, and the state words of a
 // kTcSplitF16x3 product.
 __global__ void __launch_bounds__(256)
-split_maps_kernel(const SplitProb *__restrict__ probs, int *__restrict__ unit_map,
+split_maps_kernel(const __grid_constant__ ProbTable tab, int *__restrict__ unit_map,
                   int *__restrict__ pack_map, int *__restrict__ ver_map) {
   __shared__ uint32_t mx_s[8], mn_s[8];
   const int g = blockIdx.x;
-  const SplitProb &pr = probs[g];
+  pdl_wait();
+  const SplitProb &pr = (tab.dev ? tab.dev : &tab.one)[g];
   const int units = (int)split_units(pr);
   const int packs = pr.mt * pr.kt + pr.nt * pr.kt;
   if (unit_map)
@@ -692,16 +705,15 @@ split_maps_kernel(const SplitProb *__restrict__ probs, int *__restrict__ unit_ma
 
 }  // namespace
 
-cudaError_t launch_split_maps(const SplitProb *d_probs, int nprobs, int *unit_map, int *pack_map,
-                              int *ver_map, cudaStream_t s) {
-  if (nprobs <= 0) return cudaSuccess;
+cudaError_t launch_split_maps(const ProbTable &tab, int *unit_map, int *pack_map, int *ver_map,
+                              cudaStream_t s) {
+  if (tab.n <= 0) return cudaSuccess;
   TraceScope ts("split_maps", s);
-  split_maps_kernel<<<nprobs, 256, 0, s>>>(d_probs, unit_map, pack_map, ver_map);
-  return cudaGetLastError();
+  return launch_pdl(split_maps_kernel, (unsigned)tab.n, 256, 0, s, tab, unit_map, pack_map, ver_map);
 }
 
-cudaError_t launch_split_pack(TcKind kind, int mode, const SplitProb *d_probs, int nprobs,
-                              int total_tiles, const int *map, const int *flags, int *any,
+cudaError_t launch_split_pack(TcKind kind, int mode, const ProbTable &tab, int total_tiles,
+                              const int *map, const int *flags, int *any,
                               void *pack_base, cudaStream_t s) {
   if (total_tiles <= 0) return cudaSuccess;
   TraceScope ts(mode == kPackFix ? "split_fix" : "split_pack", s);
@@ -712,47 +724,38 @@ cudaError_t launch_split_pack(TcKind kind, int mode, const SplitProb *d_probs, i
   // costs a single wave of blocks
   const int grid = mode == kPackFix ? std::min(total_tiles, sm_count() * 4) : total_tiles;
   if (kind == kTcSplitF16x3) {
-    if (mode == kPackUnscaled)
-    {
-      static std::once_flag once;
-      static cudaError_t attr_err = cudaSuccess;
-      std::call_once(once, [] {
-        attr_err = cudaFuncSetAttribute(split_pack_half_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                        kPkSmem);
-      });
-      if (attr_err != cudaSuccess) return attr_err;
-      split_pack_half_kernel<<<std::min(total_tiles, sm_count() * 2), 288, kPkSmem, s>>>(
-          d_probs, nprobs, map, any, total_tiles, pk);
-    }
-    else
-      split_fix_half_kernel<<<grid, 256, 0, s>>>(d_probs, nprobs, map, flags, any, total_tiles, pk);
-    return cudaGetLastError();
+    if (mode == kPackFix)
+      return launch_pdl(split_fix_half_kernel, (unsigned)grid, 256, 0, s, tab, map, flags,
+                        static_cast<const int *>(any), total_tiles, pk);
+    static std::once_flag once;
+    static cudaError_t attr_err = cudaSuccess;
+    std::call_once(once, [] {
+      attr_err = cudaFuncSetAttribute(split_pack_half_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                      kPkSmem);
+    });
+    if (attr_err != cudaSuccess) return attr_err;
+    return launch_pdl(split_pack_half_kernel, (unsigned)std::min(total_tiles, sm_count() * 2), 288, kPkSmem,
+                      s, tab, map, any, total_tiles, pk);
   }
-#define MM_PACK(P, M) \
-  split_pack_kernel<P, M><<<grid, 256, 0, s>>>(d_probs, nprobs, map, flags, any, total_tiles, pk)
-  if (mode == kPackUnscaled) { if (x6) MM_PACK(3, kPackUnscaled); else MM_PACK(2, kPackUnscaled); }
-  else { if (x6) MM_PACK(3, kPackFix); else MM_PACK(2, kPackFix); }
-#undef MM_PACK
-  return cudaGetLastError();
+  auto kernel = mode == kPackUnscaled ? (x6 ? split_pack_kernel<3, kPackUnscaled> : split_pack_kernel<2, kPackUnscaled>)
+                                      : (x6 ? split_pack_kernel<3, kPackFix> : split_pack_kernel<2, kPackFix>);
+  return launch_pdl_if(grid <= sm_count() * 4, kernel, (unsigned)grid, 256, 0, s, tab, map, flags,
+                       static_cast<const int *>(any), total_tiles, pk);
 }
 
-cudaError_t launch_split_verify(const SplitProb *d_probs, int nprobs, int64_t total_items,
+cudaError_t launch_split_verify(const ProbTable &tab, int64_t total_items,
                                 const int *map, int *flags, int *any, int max_kt, cudaStream_t s,
                                 bool write_cols) {
-  if (nprobs <= 0 || total_items <= 0) return cudaSuccess;
+  if (tab.n <= 0 || total_items <= 0) return cudaSuccess;
   if (total_items > 0x7fffffffLL) return cudaErrorInvalidValue;
   TraceScope ts("split_verify", s);
   const int wpi = max_kt >= 64 ? 8 : (max_kt >= 32 ? 4 : (max_kt >= 16 ? 2 : 1));
   const int ti = (int)total_items;
   const unsigned blocks = (unsigned)((total_items * wpi + 7) / 8);
-#define MM_VERIFY(W) \
-  split_verify_kernel<W><<<blocks, 256, 0, s>>>(d_probs, nprobs, map, ti, flags, any, write_cols)
-  if (wpi == 8) MM_VERIFY(8);
-  else if (wpi == 4) MM_VERIFY(4);
-  else if (wpi == 2) MM_VERIFY(2);
-  else MM_VERIFY(1);
-#undef MM_VERIFY
-  return cudaGetLastError();
+  auto kernel = wpi == 8 ? split_verify_kernel<8>
+                         : (wpi == 4 ? split_verify_kernel<4>
+                                     : (wpi == 2 ? split_verify_kernel<2> : split_verify_kernel<1>));
+  return launch_pdl(kernel, blocks, 256, 0, s, tab, map, ti, flags, any, write_cols);
 }
 
 }  // namespace mm

@@ -140,12 +140,17 @@ struct TcLayout {
   static constexpr int kSmemBytes = kStageOffset + 4 * kStageStride + 1024;  // + align slack
 };
 
-template <int BKB, int STAGES, int KIND, int MAXBN>
+// ONE: the table is one product carried in the launch (tab.one, one_cmap);
+// else dev_probs and many_cmaps.  An instantiation each: with one pointer for
+// both, the roles read a device table through generic loads again and again
+// (the FP64 emulation of 4096^3 4133 us instead of 4079).
+template <int BKB, int STAGES, int KIND, int MAXBN, bool ONE>
 __global__ void __launch_bounds__(kThreads, 1)
-tc_gemm_kernel(const __grid_constant__ CUtensorMap tmap, const SplitProb *__restrict__ probs,
-               int nprobs, const int *__restrict__ unit_map, const int *__restrict__ flags,
-               int total_units, const int *__restrict__ order, int uniform_only,
-               const CUtensorMap *__restrict__ c_maps, int *err) {
+tc_gemm_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_constant__ CUtensorMap one_cmap,
+               const __grid_constant__ ProbTable tab, const SplitProb *__restrict__ dev_probs,
+               const int *__restrict__ unit_map,
+               const int *__restrict__ flags, int total_units, const int *__restrict__ order,
+               int uniform_only, const CUtensorMap *__restrict__ many_cmaps, int *clear, int *err) {
   using L = TcLayout<BKB, STAGES, KIND, MAXBN>;
   extern __shared__ uint8_t smem_raw[];
   const uint32_t raw = smem_u32(smem_raw);
@@ -163,12 +168,11 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmap, const SplitProb *__rest
   float *stage_buf = reinterpret_cast<float *>(smem + L::kStageOffset);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  // this CTA's work units, the same sequence for every role: the host's list
-  // (grid + 1 offsets, then the units), or units c, c + grid, ...
-  const int *ulist = order ? order + gridDim.x + 1 : nullptr;
-  const int i_first = order ? order[blockIdx.x] : (int)blockIdx.x;
-  const int i_end = order ? order[blockIdx.x + 1] : total_units;
-  const int i_step = order ? 1 : (int)gridDim.x;
+  __shared__ SplitProb shared_one;
+  if (ONE) table_products(tab, &shared_one);
+  const SplitProb *__restrict__ probs = ONE ? &shared_one : dev_probs;
+  const int nprobs = ONE ? 1 : tab.n;
+  const CUtensorMap *c_maps = ONE ? &one_cmap : many_cmaps;
 
   if (warp == 0) {
     tmem_alloc(smem_u32(tmem_holder), kTmemCols);
@@ -191,6 +195,16 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmap, const SplitProb *__rest
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = *reinterpret_cast<volatile uint32_t *>(tmem_holder);
+  // the set-up above may run beside the end of the stream's previous kernel
+  pdl_wait();
+  if (clear != nullptr && blockIdx.x == 0 && threadIdx.x < kStateWords) clear[threadIdx.x] = 0;
+  // this CTA's work units, the same sequence for every role: the host's list
+  // (grid + 1 offsets, then the units), or units c, c + grid, ...
+  const int *ulist = order ? order + gridDim.x + 1 : nullptr;
+  const int i_first = order ? order[blockIdx.x] : (int)blockIdx.x;
+  const int i_end = order ? order[blockIdx.x + 1] : total_units;
+  const int i_step = order ? 1 : (int)gridDim.x;
+
 
   if (warp == 0) {
     if (lane == 0) {
@@ -612,19 +626,22 @@ cudaError_t encode_c_map(void *map, float *C, int64_t n, int64_t p) {
 
 namespace {
 
-template <int BKB, int STAGES, int KIND, int MAXBN>
-cudaError_t launch_tc_t(const SplitProb *d_probs, int nprobs, const int *unit_map,
-                        const int *flags, int total_units, void *pack_base, int64_t pack_rows,
+template <int BKB, int STAGES, int KIND, int MAXBN, bool ONE = false>
+cudaError_t launch_tc_t(const ProbTable &tab, const int *unit_map, const int *flags, int total_units, void *pack_base, int64_t pack_rows,
                         int grid, int *d_err, cudaStream_t s, const int *order,
-                        int uniform_only, const void *c_maps) {
+                        int uniform_only, const void *c_maps, int *clear) {
+  if constexpr (KIND != kTcE4m3 && !ONE)
+    if (tab.dev == nullptr)
+      return launch_tc_t<BKB, STAGES, KIND, MAXBN, true>(tab, unit_map, flags, total_units, pack_base, pack_rows,
+                                                         grid, d_err, s, order, uniform_only, c_maps, clear);
   using L = TcLayout<BKB, STAGES, KIND, MAXBN>;
-  static_assert(L::kSmemBytes <= 232448, "shared memory budget");
+  static_assert(L::kSmemBytes + sizeof(SplitProb) <= 232448, "shared memory budget");
   // one CTA per SM: the kernel allocates all 512 TMEM columns
   static_assert(2 * L::kSmemBytes > 232448, "must not fit twice on one SM");
   static std::once_flag once;
   static cudaError_t attr_err = cudaSuccess;
   std::call_once(once, [] {
-    attr_err = cudaFuncSetAttribute(tc_gemm_kernel<BKB, STAGES, KIND, MAXBN>,
+    attr_err = cudaFuncSetAttribute(tc_gemm_kernel<BKB, STAGES, KIND, MAXBN, ONE>,
                                     cudaFuncAttributeMaxDynamicSharedMemorySize, L::kSmemBytes);
   });
   if (attr_err != cudaSuccess) return attr_err;
@@ -632,10 +649,15 @@ cudaError_t launch_tc_t(const SplitProb *d_probs, int nprobs, const int *unit_ma
   cudaError_t e = encode_pack_map(&map, pack_base, pack_rows, BKB);
   if (e != cudaSuccess) return e;
   TraceScope ts(KIND == kTcE4m3 ? "fp8_tc" : "split_tc", s);
-  tc_gemm_kernel<BKB, STAGES, KIND, MAXBN><<<grid, kThreads, L::kSmemBytes, s>>>(
-      map, d_probs, nprobs, unit_map, flags, total_units, order, uniform_only,
-      static_cast<const CUtensorMap *>(c_maps), d_err);
-  return cudaGetLastError();
+  // a product carried in the launch brings its C's map along, too
+  CUtensorMap one_cmap = {};
+  if (tab.dev == nullptr && tab.one.c_tma > 0) {
+    e = encode_c_map(&one_cmap, tab.one.C, tab.one.n, tab.one.p);
+    if (e != cudaSuccess) return e;
+  }
+  return launch_pdl(tc_gemm_kernel<BKB, STAGES, KIND, MAXBN, ONE>, (unsigned)grid, kThreads, L::kSmemBytes, s,
+                    map, one_cmap, tab, tab.dev, unit_map, flags, total_units, order, uniform_only,
+                    static_cast<const CUtensorMap *>(c_maps), clear, d_err);
 }
 
 }  // namespace
@@ -738,17 +760,16 @@ size_t tc_tail_bytes(const TcTail &t, int64_t tiles, int bn) {
   return tc_tail_part_bytes(t, tiles, bn) + (((size_t)R * sizeof(int) + 255) & ~(size_t)255);
 }
 
-cudaError_t launch_tc(TcKind kind, const SplitProb *d_probs, int nprobs, int total_units,
-                      const int *unit_map, const int *flags, void *pack_base, int64_t pack_rows,
+cudaError_t launch_tc(TcKind kind, const ProbTable &tab, int total_units, const int *unit_map,
+                      const int *flags, void *pack_base, int64_t pack_rows,
                       const TcConfig &cfg, int *d_err, cudaStream_t s, const int *order,
-                      int uniform_only, const void *c_maps) {
+                      int uniform_only, const void *c_maps, int *clear) {
   if (total_units <= 0) return cudaSuccess;
   if (pack_rows <= 0 || pack_rows > 0x7fffffffLL) return cudaErrorInvalidValue;
   const int grid = tc_launch_grid(cfg, total_units);
   const int *mp = unit_map;
 #define MM_TC_ARGS \
-  d_probs, nprobs, mp, flags, total_units, pack_base, pack_rows, grid, d_err, s, order, \
-      uniform_only, c_maps
+  tab, mp, flags, total_units, pack_base, pack_rows, grid, d_err, s, order, uniform_only, c_maps, clear
   cudaError_t e = cudaErrorInvalidValue;
   const bool narrow = cfg.max_bn <= 128;  // every N tile of the table fits 128
   if (kind == kTcE4m3) e = launch_tc_t<128, 4, kTcE4m3, 256>(MM_TC_ARGS);

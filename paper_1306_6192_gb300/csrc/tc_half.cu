@@ -15,8 +15,9 @@
 // 128 x 128 tile then holds 256 columns, so two tiles fit tensor memory and a
 // tile's epilogue runs beside the next one's MMAs.  The main accumulator
 // takes a sixth of the additions of the bf16 form.  The tensor cores' FP32 sums
-// are not rounded to nearest, so a long sum of one sign drifts; every 512 K the
-// accumulator is therefore handed to the epilogue warps, which add the
+// are not rounded to nearest, so a long sum of one sign drifts; every 512 K (256
+// for products that the fused kernel's shorter sums served before; chunk, K
+// blocks) the accumulator is therefore handed to the epilogue warps, which add the
 // chunks in registers with round-to-nearest additions beside the next chunk's
 // MMAs (2048^3, max error over |A||B|: signed entries 1.2e-7 against 2.0e-6 for the
 // six bf16 products, entries in [0, 1) 3.0e-6 against 1.2e-5).
@@ -75,7 +76,6 @@ constexpr int kPart6 = 128 * 64;         // three-part form: 64 bytes of K
 constexpr int kStageBytes6 = 6 * kPart6;
 static_assert(kStageBytes6 <= kStageBytes, "the three-part form fits the stage");
 constexpr int kAccs = 2, kAccCols = 256;
-constexpr int kChunk = 8;                // K blocks summed in one accumulator
 constexpr int kUnits = 4;                // descriptor ring
 constexpr int kEpiWarps = kHalfSplitCnt, kEpiThreads = 32 * kEpiWarps;
 constexpr int kFirstEpi = 4;             // warp 3 idles: whole warpgroups share registers
@@ -96,7 +96,7 @@ struct __align__(16) Unit {
   int32_t k0, k1;      // stages; k1 < 0: no more units
   int32_t x6, ex;      // three-part form; fp16 form: exponent of the result
   int32_t n, p, row0, col0;
-  int32_t flags, vec8, split_s, h, epi_on;
+  int32_t flags, vec8, split_s, h, epi_on, chunk;
   float alpha, beta;
 };
 static_assert(sizeof(Unit) <= 128, "descriptor slot");
@@ -112,7 +112,7 @@ static constexpr int kBarOff = kColOff + kEpiWarps * 64 * 2;
   static constexpr int kMiscOff = kBarOff + kNumBars * 8;
   static constexpr int kSmem = kMiscOff + 32 + 1024;          // + alignment slack
 };
-static_assert(Lay::kSmem <= 232448, "shared memory budget");
+static_assert(Lay::kSmem + sizeof(SplitProb) <= 232448, "shared memory budget");
 
 // mbar_wait with its slow path in line: a call would spill the epilogue's sums
 // around it.
@@ -148,8 +148,9 @@ __device__ __forceinline__ uint32_t idesc_f16(uint32_t fmt, int bn) {
 __global__ void __launch_bounds__(kThreads, 1)
 tc_half_kernel(const __grid_constant__ CUtensorMap map, const __grid_constant__ CUtensorMap map6,
                const __grid_constant__ CUtensorMap map_d,
-               const SplitProb *__restrict__ probs, int nprobs, const int *__restrict__ unit_map,
-               const int *__restrict__ flags, int total_units, const int *__restrict__ order, int *err) {
+               const __grid_constant__ ProbTable tab, const int *__restrict__ unit_map,
+               const int *__restrict__ flags, int total_units, const int *__restrict__ order, int *clear,
+               int *err) {
   extern __shared__ uint8_t smem_raw[];
   const uint32_t raw = smem_u32(smem_raw);
   const uint32_t sbase = (raw + 1023u) & ~1023u;
@@ -168,6 +169,9 @@ tc_half_kernel(const __grid_constant__ CUtensorMap map, const __grid_constant__ 
   auto unit_at = [&](int u) { return reinterpret_cast<Unit *>(reinterpret_cast<uint8_t *>(units) + 128 * u); };
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  __shared__ SplitProb shared_one;
+  const SplitProb *probs = table_products(tab, &shared_one);
+  const int nprobs = tab.n;
 
   if (warp == 0) {
     tmem_alloc(smem_u32(tmem_holder), kAccs * kAccCols);
@@ -196,6 +200,9 @@ tc_half_kernel(const __grid_constant__ CUtensorMap map, const __grid_constant__ 
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = *reinterpret_cast<volatile uint32_t *>(tmem_holder);
+  // the set-up above may run beside the end of the stream's previous kernel
+  pdl_wait();
+  if (clear != nullptr && blockIdx.x == 0 && threadIdx.x < kStateWords) clear[threadIdx.x] = 0;
 
   if (warp < kFirstEpi) {
     asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kRoleRegs));
@@ -255,13 +262,13 @@ tc_half_kernel(const __grid_constant__ CUtensorMap map, const __grid_constant__ 
             break;
           }
           const Unit *d = unit_at(us);
-          const int k0 = d->k0, k1 = d->k1, x6 = d->x6;
+          const int k0 = d->k0, k1 = d->k1, x6 = d->x6, in_chunk = d->chunk - 1;
           mbar_arrive(unite_bar(us));
           if (++us == kUnits) us = 0, uphase ^= 1u;
           if (k1 < 0) break;
           uint32_t t0 = 0;
           for (int ki = k0; ki < k1; ki++) {
-            const bool first = ki == k0 || (!x6 && (ki - k0) % kChunk == 0);
+            const bool first = ki == k0 || (!x6 && ((ki - k0) & in_chunk) == 0);
             if (first) {
               // the accumulator of the last chunk goes to the epilogue
               if (ki != k0) {
@@ -355,6 +362,7 @@ tc_half_kernel(const __grid_constant__ CUtensorMap map, const __grid_constant__ 
           d.sA = pr.sA;
           d.tB = pr.tB;
           d.split_s = pr.split_s;
+          d.chunk = pr.chunk;
           d.h = tc.h;
           const int st = tc.t - pr.split_from;
           d.part = tc.h >= 0 ? pr.part + (size_t)st * pr.split_s * (kTcBM * kBN) : nullptr;
@@ -411,7 +419,7 @@ tc_half_kernel(const __grid_constant__ CUtensorMap map, const __grid_constant__ 
       if (d->k1 < 0) break;
       const int n = d->n, p = d->p, x6 = d->x6, h = d->h, split_s = d->split_s, epi_on = d->epi_on;
       const int row0 = d->row0 + q * 32, col0 = d->col0;
-      const int chunks = x6 ? 1 : (d->k1 - d->k0 + kChunk - 1) / kChunk;
+      const int chunks = x6 ? 1 : (d->k1 - d->k0 + d->chunk - 1) / d->chunk;
       // whole 32-byte sectors: C (and D) 32-byte aligned, p % 8 == 0
       const bool vec8 = d->vec8 != 0;
       const bool vec_d = vec8 && epi_on == 2;
@@ -654,10 +662,10 @@ tc_half_kernel(const __grid_constant__ CUtensorMap map, const __grid_constant__ 
 
 }  // namespace
 
-cudaError_t launch_tc_half(const SplitProb *d_probs, int nprobs, int total_units,
+cudaError_t launch_tc_half(const ProbTable &tab, int total_units,
                            const int *unit_map, const int *flags, void *pack_base,
                            int64_t pack_rows, int grid, int *d_err, cudaStream_t s,
-                           const int *order, const SplitProb *with_d) {
+                           const int *order, int *clear) {
   // one CTA per SM: the kernel allocates all 512 TMEM columns
   static_assert(2 * Lay::kSmem > 232448, "must not fit twice on one SM");
   static std::once_flag once;
@@ -669,13 +677,14 @@ cudaError_t launch_tc_half(const SplitProb *d_probs, int nprobs, int total_units
   CUtensorMap map, map6, map_d = {};
   cudaError_t e = encode_pack_map(&map, pack_base, pack_rows, 128, 256);
   if (e == cudaSuccess) e = encode_pack_map(&map6, pack_base, pack_rows, 64, 128);
-  if (e == cudaSuccess && with_d && tc_c_map_ok(with_d->epi.D, with_d->n, with_d->p))
-    e = encode_c_map(&map_d, const_cast<float *>(with_d->epi.D), with_d->n, with_d->p);
+  // (only a product of its own has an epilogue)
+  const SplitProb &one = tab.one;
+  if (e == cudaSuccess && tab.dev == nullptr && one.epi.on == 2 && tc_c_map_ok(one.epi.D, one.n, one.p))
+    e = encode_c_map(&map_d, const_cast<float *>(one.epi.D), one.n, one.p);
   if (e != cudaSuccess) return e;
   TraceScope ts("split_tc", s);
-  tc_half_kernel<<<grid, kThreads, Lay::kSmem, s>>>(map, map6, map_d, d_probs, nprobs, unit_map, flags,
-                                                    total_units, order, d_err);
-  return cudaGetLastError();
+  return launch_pdl(tc_half_kernel, (unsigned)grid, kThreads, Lay::kSmem, s, map, map6, map_d, tab, unit_map,
+                    flags, total_units, order, clear, d_err);
 }
 
 }  // namespace mm

@@ -42,7 +42,7 @@ TcTail plan_tail(SplitProb &sp, TcKind kind, const TcChoice &ch) {
 }
 
 mm_status run_tc_groups(Scratch &ws, const mm_problem *probs, int count, cudaStream_t s,
-                        const TcChoice *force, bool six, const Epi *epi) {
+                        const TcChoice *force, bool six, const Epi *epi, int chunk) {
   Group groups[2] = {{kTcSplitBf16x3}, {six ? kTcSplitBf16x6 : kTcSplitF16x3}};
   int64_t rows = 0, scal = 0, part = 0, half = 0;
   size_t tail_parts = 0, tail_cnts = 0;  // partial tiles and counters of tail splits
@@ -92,6 +92,7 @@ mm_status run_tc_groups(Scratch &ws, const mm_problem *probs, int count, cudaStr
     part += (int64_t)sp.kt * q.p;
     // state words of the fp16 kind (offset + 1, fixed below)
     if (kind == kTcSplitF16x3) sp.hx = reinterpret_cast<int32_t *>((uintptr_t)(++half));
+    sp.chunk = chunk;
     sp.ver_start = (int32_t)G.vers;
     G.vers += verify_items(q.n, q.p);
     G.max_kt = std::max(G.max_kt, sp.kt);
@@ -171,19 +172,36 @@ mm_status run_tc_groups(Scratch &ws, const mm_problem *probs, int count, cudaStr
       }
       all.push_back(sp);
     }
+  // a table of one product travels in the launches, and its state words and
+  // tail counters in words that are zero between calls: nothing to copy or to
+  // set ahead of its kernels
+  const bool single = ntab == 1;
+  int *state = nullptr, *clear = nullptr;
+  if (single) {
+    SplitProb &sp = all[0];
+    if ((e = ws.take_words(tail_cnts, s, &state, &clear)) != cudaSuccess) return note_cuda(e);
+    if (sp.hx) sp.hx = state + kStateHalf;
+    if (sp.split_s > 1) sp.cnt = ws.counters();
+  }
   SplitProb *d_tab = reinterpret_cast<SplitProb *>(base + tab_off);
   int *d_orders = reinterpret_cast<int *>(base + tab_off + tab_bytes);
   const void *d_cmaps = cmap_bytes ? static_cast<const void *>(base + tab_off + cmap_rel) : nullptr;
-  {
+  // C matrices that the tensor-core kernel may write with tiled stores
+  auto tiled_c = [](const SplitProb &sp) {
+    // the epilogue C = alpha (A.B) + beta D loads D in 16-byte vectors beside
+    // the tiled stores (a D off that alignment: plain stores); tc_half.cu
+    // stores whole sectors from registers
+    return sp.hx == nullptr && (sp.epi.on != 2 || (reinterpret_cast<uintptr_t>(sp.epi.D) & 15u) == 0) &&
+           tc_c_map_ok(sp.C, sp.n, sp.p);
+  };
+  if (single) {
+    all[0].c_tma = tiled_c(all[0]) ? 1 : 0;
+  } else {
     // one copy: the table, the CTAs' unit lists, the C tensor maps
     std::vector<uint8_t> blob(cmap_rel + cmap_bytes, 0);
     for (size_t k = 0; cmap_bytes && k < ntab; k++) {
       SplitProb &sp = all[k];
-      if (sp.hx) continue;  // tc_half.cu stores whole sectors from registers
-      // the epilogue C = alpha (A.B) + beta D loads D in 16-byte vectors
-      // beside the tiled stores (a D off that alignment: plain stores)
-      const bool d_ok = sp.epi.on != 2 || (reinterpret_cast<uintptr_t>(sp.epi.D) & 15u) == 0;
-      if (d_ok && tc_c_map_ok(sp.C, sp.n, sp.p) &&
+      if (tiled_c(sp) &&
           encode_c_map(blob.data() + cmap_rel + k * kMapBytes, sp.C, sp.n, sp.p) == cudaSuccess)
         sp.c_tma = (int32_t)k + 1;
     }
@@ -195,20 +213,19 @@ mm_status run_tc_groups(Scratch &ws, const mm_problem *probs, int count, cudaStr
       at += o.size() * sizeof(int);
     }
     e = ws.stage.copy_to_device(d_tab, blob.data(), blob.size(), s);
+    if (e == cudaSuccess) e = cudaMemsetAsync(base + scal_off, 0, zero_end - scal_off, s);
+    if (e != cudaSuccess) return note_cuda(e);
   }
-  if (e != cudaSuccess) return note_cuda(e);
-  e = cudaMemsetAsync(base + scal_off, 0, zero_end - scal_off, s);
-  if (e != cudaSuccess) return note_cuda(e);
   size_t off = 0;
   int *flags_all = reinterpret_cast<int *>(base + flag_off);
   int *maps = reinterpret_cast<int *>(base + map_off);
   for (int gi = 0; gi < 2; gi++) {
     Group &G = groups[gi];
     if (G.tab.empty()) continue;
-    const SplitProb *dt = d_tab + off;
-    int *flags = flags_all + off;
-    int *any = flags_all + ntab + gi;
     const int np = (int)G.tab.size();
+    const ProbTable dt = single ? ProbTable{nullptr, 1, all[0]} : device_table(d_tab + off, np);
+    int *flags = single ? state + kStateFlags : flags_all + off;
+    int *any = single ? state + kStateAny : flags_all + ntab + gi;
     off += G.tab.size();
     int *tile_map = nullptr, *pack_map = nullptr, *ver_map = nullptr;
     const int *order = nullptr;
@@ -221,25 +238,27 @@ mm_status run_tc_groups(Scratch &ws, const mm_problem *probs, int count, cudaStr
       pack_map = tile_map + G.units;
       ver_map = pack_map + G.packs;
       maps = ver_map + G.vers;
-      e = launch_split_maps(dt, np, tile_map, pack_map, ver_map, s);
+      e = launch_split_maps(dt, tile_map, pack_map, ver_map, s);
       if (e != cudaSuccess) return note_cuda(e);
     }
 
     // one unscaled pass that also reduces the maxima, then the operands out
     // of range are re-packed with their scales
-    e = launch_split_pack(G.kind, kPackUnscaled, dt, np, (int)G.packs, pack_map, nullptr, any,
+    e = launch_split_pack(G.kind, kPackUnscaled, dt, (int)G.packs, pack_map, nullptr, any,
                           base, s);
-    if (e == cudaSuccess) e = launch_split_verify(dt, np, G.vers, ver_map, flags, any, G.max_kt, s);
+    if (e == cudaSuccess) e = launch_split_verify(dt, G.vers, ver_map, flags, any, G.max_kt, s);
     if (e == cudaSuccess)
-      e = launch_split_pack(G.kind, kPackFix, dt, np, (int)G.packs, pack_map, flags, any, base, s);
+      e = launch_split_pack(G.kind, kPackFix, dt, (int)G.packs, pack_map, flags, any, base, s);
     if (e == cudaSuccess)
       e = G.kind == kTcSplitF16x3
-              ? launch_tc_half(dt, np, (int)G.units, tile_map, flags, base, rows,
-                               tc_launch_grid(G.cfg, G.units), g_ctx.d_err, s, order,
-                               G.tab[0].epi.on == 2 ? &G.tab[0] : nullptr)
-              : launch_tc(G.kind, dt, np, (int)G.units, tile_map, flags, base, rows, G.cfg, g_ctx.d_err,
-                          s, order, 0, d_cmaps);
-    if (e != cudaSuccess) return note_cuda(e);
+              ? launch_tc_half(dt, (int)G.units, tile_map, flags, base, rows,
+                               tc_launch_grid(G.cfg, G.units), g_ctx.d_err, s, order, clear)
+              : launch_tc(G.kind, dt, (int)G.units, tile_map, flags, base, rows, G.cfg, g_ctx.d_err,
+                          s, order, 0, d_cmaps, clear);
+    if (e != cudaSuccess) {
+      ws.words_epoch = 0;  // the words may be left set
+      return note_cuda(e);
+    }
   }
   return MM_OK;
 }
@@ -324,25 +343,25 @@ mm_status run_split_chunked(Scratch &ws, int64_t n, int64_t m, int64_t p, const 
   for (int c = 0; c < chunks; c++) {
     if (c == 0 && (e = cudaStreamWaitEvent(s, in_ready[0], 0)) != cudaSuccess) break;
     if ((e = cudaStreamWaitEvent(s, in_ready[c + 1], 0)) != cudaSuccess) break;
-    const SplitProb *dt = d_tab + c;
+    const ProbTable dt = device_table(d_tab + c, 1);
     int *flag = reinterpret_cast<int *>(base + flag_off) + c;
     int *any = flag + chunks;
     // slab 0 packs (and reduces) B as well; a later slab's verify sees all of
     // B's column maxima, so its B flag equals slab 0's, and it leaves B's
     // column words (read by the GEMMs in flight) untouched
-    if ((e = launch_split_pack(kind, kPackUnscaled, dt, 1, (int)packs[(size_t)c], nullptr, nullptr,
+    if ((e = launch_split_pack(kind, kPackUnscaled, dt, (int)packs[(size_t)c], nullptr, nullptr,
                                nullptr, base, s)) != cudaSuccess)
       break;
-    if ((e = launch_split_verify(dt, 1, verify_items(tab[(size_t)c].n, p), nullptr, flag, any, kt,
+    if ((e = launch_split_verify(dt, verify_items(tab[(size_t)c].n, p), nullptr, flag, any, kt,
                                  s, c == 0)) != cudaSuccess)
       break;
-    if ((e = launch_split_pack(kind, kPackFix, dt, 1, (int)packs[(size_t)c], nullptr, flag, any,
+    if ((e = launch_split_pack(kind, kPackFix, dt, (int)packs[(size_t)c], nullptr, flag, any,
                                base, s)) != cudaSuccess)
       break;
     if ((e = cudaEventRecord(g_ctx.ev_prep[c], s)) != cudaSuccess) break;
     cudaStream_t t = g_ctx.tc_streams[c & 1];
     if ((e = cudaStreamWaitEvent(t, g_ctx.ev_prep[c], 0)) != cudaSuccess) break;
-    if ((e = launch_tc(kind, dt, 1, (int)tiles[(size_t)c], nullptr, flag, base, rows, cfg,
+    if ((e = launch_tc(kind, dt, (int)tiles[(size_t)c], nullptr, flag, base, rows, cfg,
                        g_ctx.d_err, t)) != cudaSuccess)
       break;
     if ((e = cudaEventRecord(out_ready[c], t)) != cudaSuccess) break;
@@ -353,8 +372,8 @@ mm_status run_split_chunked(Scratch &ws, int64_t n, int64_t m, int64_t p, const 
 }
 
 mm_status run_split(Scratch &ws, const mm_problem *probs, int count, cudaStream_t s,
-                    const TcChoice *force, bool six, const Epi *epi) {
-  return run_tc_groups(ws, probs, count, s, force, six, epi);
+                    const TcChoice *force, bool six, const Epi *epi, int chunk) {
+  return run_tc_groups(ws, probs, count, s, force, six, epi, chunk);
 }
 
 mm_status run_fp8(Scratch &ws, const mm_problem *probs, int count, cudaStream_t s) {
