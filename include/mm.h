@@ -412,7 +412,7 @@ mm_status mm_measure_fma_peak(mm_dtype dt, int64_t iters, double *flops_per_s);
  * time (ms) of the kernel named `kernel` ("simt_f32", "dgemm_f64", "simt_sum" (the
  * fixed-order sum of a K-sliced SIMT or FP64 product), "split_maps", "split_pack",
  * "split_verify", "split_fix", "split_tc", "fused_tc", "fp8_max", "fp8_pack", "fp8_tc",
- * "fp8_blk", "check_f64", "ozaki_max", "ozaki_map", "ozaki_digits", "ozaki_sum",
+ * "fp8_blk", "check_f64", "ozaki_max", "ozaki_digits", "ozaki_sum",
  * "ozaki_gate", "add", "diag", "cplx_planes", "cplx_combine") since the last reset.
  * Reading synchronises the recorded events. */
 mm_status mm_trace_enable(int on);

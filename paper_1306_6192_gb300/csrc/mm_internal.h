@@ -355,6 +355,17 @@ struct TraceScope {
 int sm_count();
 
 #ifdef __CUDACC__
+inline void pdl_config(cudaLaunchConfig_t &cfg, cudaLaunchAttribute (&at)[1], dim3 grid, unsigned block,
+                       size_t smem, cudaStream_t s) {
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3(block, 1, 1);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+}
 // Launch as a programmatic dependent of the stream's previous kernel: the
 // blocks may become resident while that kernel finishes.  The kernel calls
 // pdl_wait() in every block before it touches global memory that earlier work
@@ -367,14 +378,8 @@ template <typename... KArgs, typename... Args>
 cudaError_t launch_pdl_if(bool dependent, void (*kernel)(KArgs...), unsigned grid, unsigned block,
                           size_t smem, cudaStream_t s, Args... args) {
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(grid, 1, 1);
-  cfg.blockDim = dim3(block, 1, 1);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = s;
   cudaLaunchAttribute at[1];
-  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  at[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = at;
+  pdl_config(cfg, at, dim3(grid, 1, 1), block, smem, s);
   cfg.numAttrs = dependent ? 1 : 0;
   return cudaLaunchKernelEx(&cfg, kernel, args...);
 }

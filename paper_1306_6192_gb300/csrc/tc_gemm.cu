@@ -655,8 +655,10 @@ cudaError_t launch_tc_t(const ProbTable &tab, const int *unit_map, const int *fl
     e = encode_c_map(&one_cmap, tab.one.C, tab.one.n, tab.one.p);
     if (e != cudaSuccess) return e;
   }
-  return launch_pdl(tc_gemm_kernel<BKB, STAGES, KIND, MAXBN, ONE>, (unsigned)grid, kThreads, L::kSmemBytes, s,
-                    map, one_cmap, tab, tab.dev, unit_map, flags, total_units, order, uniform_only,
+  // (as a dependent of the digit kernel the FP64 emulation's launch made its call
+  // 2.5% slower, 4090 us against 3990 at 4096^3)
+  return launch_pdl_if(ONE, tc_gemm_kernel<BKB, STAGES, KIND, MAXBN, ONE>, (unsigned)grid, kThreads,
+                       L::kSmemBytes, s, map, one_cmap, tab, tab.dev, unit_map, flags, total_units, order, uniform_only,
                     static_cast<const CUtensorMap *>(c_maps), clear, d_err);
 }
 
