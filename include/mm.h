@@ -374,7 +374,7 @@ mm_status mm_tune_query_splitk(int64_t n, int64_t m, int64_t p, int *tiles, int 
  * 64 x 64 in FP64) than half the SMs is cut along K into *slices slices of
  * *slice_k values (the last one shorter), computed on *tile x *tile output
  * tiles (64, or 128 for FP32 products at least 128 wide both ways;
- * FP64 tiles may run as four quarters, to the same bits); the
+ * a kernel may cut them into smaller ones, to the same bits); the
  * slices' partial sums are then added in a fixed order.  The plan keeps one
  * wave of at most two CTAs per SM, slices of at least 128 values unless K is
  * shorter, and partials of at most 256 MiB; it depends on the shape (and

@@ -10,11 +10,11 @@
 //
 // Every output is accumulated by one thread with r ascending, as in the
 // definition of the Cauchy product.  Products with too few output tiles to
-// fill the SMs (skinny ones above all) are cut along K into S slices (64 x 64
-// tiles, or 128 x 128 for FP32 products at least 128 wide both ways): each
+// fill the SMs (skinny ones above all) are cut along K into S slices: each
 // slice's partial product in that order, then the S
 // partials of each entry added in a fixed grouping and order by a second
-// kernel.
+// kernel or within a cluster of blocks.  The tiles (128, 64 or 32 in FP32, 64 or 32 in
+// FP64) change no sum.
 #include <algorithm>
 #include <type_traits>
 
@@ -389,6 +389,230 @@ cudaError_t launch_splitk(int64_t n, int64_t m, int64_t p, const T *A, const T *
                           static_cast<const T *>(part), pl.S, np, C, run_if, ep);
 }
 
+// Small FP32 tiles: BM x BN outputs, TM x 4 a thread, a warp 4 TM x 32.  The
+// operands come by cp.async into a ring of kRingStages K blocks, all of them in
+// flight at once, A as it lies (rows padded to keep four neighbouring rows on
+// different banks; a thread takes its rows four apart) and read four k at a
+// time; every output is accumulated with r ascending, as in simt_tile: the same bits.
+// Up to kSimtCluster slices of K are a cluster, which adds the slices'
+// partials in the sum kernel's order through shared memory; more of them write
+// `out` + z n p for that kernel.
+constexpr int kRingStages = 4, kSimtCluster = 8;
+
+template <int BM, int BN, int TM>
+struct RingShape {
+  static constexpr int BK = BM == 32 ? 32 : 16;
+  static constexpr int LDA = BK + 4;
+  static constexpr int NT = (BM / (4 * TM)) * (BN / 32) * 32;
+  static constexpr int kStage = BM * LDA + BK * BN;  // floats
+  static_assert(kRingStages * kStage * 4 <= 48 * 1024, "static shared memory");
+  static_assert(BM * BN <= kRingStages * kStage, "the partial tile fits the ring");
+};
+
+// W floats to shared memory: a copy in flight, or zeros outside the matrix.
+template <int W>
+__device__ __forceinline__ void copy_or_zero(uint32_t dst, const float *src, bool live) {
+  if (W == 4) {
+    if (live)
+      asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
+    else
+      asm volatile("st.shared.v4.f32 [%0], {%1, %1, %1, %1};" ::"r"(dst), "f"(0.0f) : "memory");
+  } else {
+    if (live)
+      asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(dst), "l"(src) : "memory");
+    else
+      asm volatile("st.shared.f32 [%0], %1;" ::"r"(dst), "f"(0.0f) : "memory");
+  }
+}
+
+template <int BM, int BN, int TM, bool VEC, bool EPI>
+__global__ void __launch_bounds__(RingShape<BM, BN, TM>::NT)
+simt_ring_kernel(const float *__restrict__ A, const float *__restrict__ B, OutPtr<float, EPI> out, int64_t n,
+                 int64_t m, int64_t p, int64_t ks, int cluster, bool early, EpiT<float> epi) {
+  using R = RingShape<BM, BN, TM>;
+  constexpr int BK = R::BK, LDA = R::LDA, NT = R::NT;
+  __shared__ __align__(16) float ring[kRingStages * R::kStage];
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  if (early) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int64_t m0 = (int64_t)blockIdx.y * BM, n0 = (int64_t)blockIdx.x * BN;
+  const int64_t kz = (int64_t)blockIdx.z * ks, kend = min(kz + ks, m);
+  const int kblocks = (int)((kend - kz + BK - 1) / BK);
+  const uint32_t ring0 = (uint32_t)__cvta_generic_to_shared(ring);
+
+  auto load_block = [&](int kb) {
+    if (kb < kblocks) {
+      const uint32_t as = ring0 + (uint32_t)(kb % kRingStages) * R::kStage * 4, bs = as + BM * LDA * 4;
+      const int64_t k0 = kz + (int64_t)kb * BK;
+      constexpr int W = VEC ? 4 : 1;
+#pragma unroll
+      for (int i = 0; i < BM * BK / W / NT; i++) {
+        const int v = tid + i * NT, r = v / (BK / W), c = (v % (BK / W)) * W;
+        const bool live = m0 + r < n && k0 + c < kend;
+        copy_or_zero<W>(as + (r * LDA + c) * 4, A + (m0 + r) * m + k0 + c, live);
+      }
+#pragma unroll
+      for (int i = 0; i < BK * BN / W / NT; i++) {
+        const int v = tid + i * NT, r = v / (BN / W), c = (v % (BN / W)) * W;
+        const bool live = k0 + r < kend && n0 + c < p;
+        copy_or_zero<W>(bs + (r * BN + c) * 4, B + (k0 + r) * p + n0 + c, live);
+      }
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+  for (int kb = 0; kb < kRingStages; kb++) load_block(kb);
+
+  const int tx = lane & 7, ty = lane >> 3;
+  const int row0 = (warp / (BN / 32)) * (4 * TM) + ty, col0 = (warp % (BN / 32)) * 32 + tx * 4;
+  float acc[TM][4];
+#pragma unroll
+  for (int i = 0; i < TM; i++)
+#pragma unroll
+    for (int j = 0; j < 4; j++) acc[i][j] = 0.0f;
+  for (int kb = 0; kb < kblocks; kb++) {
+    asm volatile("cp.async.wait_group %0;" ::"n"(kRingStages - 1) : "memory");
+    __syncthreads();
+    const float *as = ring + (kb % kRingStages) * R::kStage, *bs = as + BM * LDA;
+#pragma unroll
+    for (int k = 0; k < BK; k += 4) {
+      float a[TM][4];
+#pragma unroll
+      for (int i = 0; i < TM; i++)
+        *reinterpret_cast<float4 *>(a[i]) = *reinterpret_cast<const float4 *>(as + (row0 + 4 * i) * LDA + k);
+#pragma unroll
+      for (int e = 0; e < 4; e++) {
+        float b[4];
+        *reinterpret_cast<float4 *>(b) = *reinterpret_cast<const float4 *>(bs + (k + e) * BN + col0);
+#pragma unroll
+        for (int i = 0; i < TM; i++)
+#pragma unroll
+          for (int j = 0; j < 4; j++) acc[i][j] = fmaf(a[i][e], b[j], acc[i][j]);
+      }
+    }
+    if (kb + kRingStages < kblocks) __syncthreads();  // the stage's readers are done
+    load_block(kb + kRingStages);
+  }
+
+  if (!early) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+
+  auto put = [&](float *C, int64_t row, int64_t col, float4 v, bool apply) {
+    if (row >= n || col >= p) return;
+    const int64_t x = row * p + col;
+    float t[4] = {v.x, v.y, v.z, v.w};
+    if (VEC) {
+#pragma unroll
+      for (int e = 0; e < 4; e++) t[e] = EPI && apply ? epi_apply(epi, t[e], x + e) : t[e];
+      *reinterpret_cast<float4 *>(C + x) = make_float4(t[0], t[1], t[2], t[3]);
+    } else {
+#pragma unroll
+      for (int e = 0; e < 4; e++)
+        if (col + e < p) C[x + e] = EPI && apply ? epi_apply(epi, t[e], x + e) : t[e];
+    }
+  };
+  if (cluster <= 1) {
+    // one slice (the epilogue's), or partials that the sum kernel adds
+    float *C = out + (int64_t)blockIdx.z * n * p;
+#pragma unroll
+    for (int i = 0; i < TM; i++)
+      put(C, m0 + row0 + 4 * i, n0 + col0, make_float4(acc[i][0], acc[i][1], acc[i][2], acc[i][3]), true);
+    return;
+  }
+  __syncthreads();
+#pragma unroll
+  for (int i = 0; i < TM; i++)
+    *reinterpret_cast<float4 *>(ring + (row0 + 4 * i) * BN + col0) =
+        make_float4(acc[i][0], acc[i][1], acc[i][2], acc[i][3]);
+  asm volatile("barrier.cluster.arrive.release;\nbarrier.cluster.wait.acquire;" ::: "memory");
+  for (int v = (int)blockIdx.z * NT + tid; v < BM * BN / 4; v += cluster * NT) {
+    float4 sum;
+    for (int s = 0; s < cluster; s++) {
+      uint32_t addr;
+      float4 t;
+      asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(addr) : "r"(ring0 + 16u * v), "r"(s));
+      asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];"
+                   : "=f"(t.x), "=f"(t.y), "=f"(t.z), "=f"(t.w)
+                   : "r"(addr));
+      sum = s == 0 ? t : make_float4(sum.x + t.x, sum.y + t.y, sum.z + t.z, sum.w + t.w);
+    }
+    put(out, m0 + v / (BN / 4), n0 + (v % (BN / 4)) * 4, sum, true);
+  }
+  // the partials stay until every block of the cluster has read them
+  asm volatile("barrier.cluster.arrive.release;\nbarrier.cluster.wait.acquire;" ::: "memory");
+}
+
+bool f32_vec(const float *A, const float *B, const float *out, int64_t m, int64_t p) {
+  return aligned16(A) && aligned16(B) && aligned16(out) && m % 4 == 0 && p % 4 == 0;
+}
+
+template <int BM, int BN, int TM>
+cudaError_t launch_ring(int64_t n, int64_t m, int64_t p, const float *A, const float *B, float *C, float *part,
+                        int S, int64_t ks, cudaStream_t s, const Epi *epi) {
+  using R = RingShape<BM, BN, TM>;
+  const int64_t gy = ceil_div(n, BM), gx = ceil_div(p, BN);
+  if (gy > 65535 || gx > 2147483647LL || S < 1 || S > 65535) return cudaErrorInvalidValue;
+  const bool clustered = S > 1 && S <= kSimtCluster;
+  float *out = S > 1 && !clustered ? part : C;
+  if (out == nullptr) return cudaErrorInvalidValue;
+  const bool vec = f32_vec(A, B, out, m, p);
+  const EpiT<float> ep = epi_of<float>(epi);
+  const EpiT<float> none{nullptr, 1.0f, 0.0f, 0};
+  const bool use = ep.on != 0 && out == C;
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute at[2];
+  cfg.gridDim = dim3((unsigned)gx, (unsigned)gy, (unsigned)S);
+  cfg.blockDim = dim3(R::NT, 1, 1);
+  cfg.stream = s;
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  at[1].id = cudaLaunchAttributeClusterDimension;
+  at[1].val.clusterDim = {1, 1, (unsigned)S};
+  cfg.attrs = at;
+  cfg.numAttrs = clustered ? 2 : 1;
+  // Dependents become resident early only behind short kernels: their blocks, waiting, take
+  // the slots where a SM has a tile less to do, and the next product then runs
+  // unevenly (1280^3, a call after another: 178 us, 111 with the trigger late),
+  // against about 3 us for the gap (512^3: 14.6 us late, 11.2 early).
+  const bool early = ceil_div(gx * gy * S, sm_count()) * BM * BN * ks <= 12000 * 128;
+  cudaError_t e;
+  {
+    TraceScope ts("simt_f32", s);
+    auto launch = [&](auto kernel) {
+      return cudaLaunchKernelEx(&cfg, kernel, A, B, out, n, m, p, ks, clustered ? S : 1, early, use ? ep : none);
+    };
+    if (use)
+      e = vec ? launch(simt_ring_kernel<BM, BN, TM, true, true>) : launch(simt_ring_kernel<BM, BN, TM, false, true>);
+    else
+      e = vec ? launch(simt_ring_kernel<BM, BN, TM, true, false>) : launch(simt_ring_kernel<BM, BN, TM, false, false>);
+  }
+  if (e != cudaSuccess || out == C) return e;
+  TraceScope ts("simt_sum", s);
+  const int64_t np = n * p;
+  if (ceil_div(np, 32) > 2147483647LL) return cudaErrorInvalidValue;
+  return launch_dependent(splitk_sum_kernel<float>, dim3((unsigned)ceil_div(np, 32), 1, 1), s,
+                          static_cast<const float *>(part), S, np, C, static_cast<const int *>(nullptr), ep);
+}
+
+// The tile of an FP32 product in S slices of K.  The CUDA cores bound it, so
+// its time goes with the work of the busiest SM: rounds of tiles times the
+// tile's outputs, weighed by what an output costs in each kernel on a full chip
+// (GB300, us for 128 / 64 / 32: 2048^3 359 / 393 / 427; with 4-byte copies,
+// 2047 x 2047 x 2045, 423 / 521 / 670).  A 128 x 128 tile takes 8 us for every 128 k
+// however small the product, so slices of it go to small tiles wherever
+// a cluster adds them (256^3, 8 tiles of 128 on 152 SMs, and their sum 16.7 / 8.0 /
+// 5.1; 768^3 45 / 26 / 32; 1024^3 81 / 57 / 63); beyond that the work decides
+// (256 x 1500 x 512 22 / 33 / 21; 512 x 4096 x 512 54 / 65 / 71), as in one pass (1152^3 111 /
+// 103 / 93; 1280^3 123 / 114 / 122; 1536^3 147 / 177 / 196).  One 64 x 64 tile a
+// SM has too few warps (48 x 700 x 1900 12 / 16 / 12).
+int f32_tile(int64_t n, int64_t p, int64_t S, bool vec, bool small_only) {
+  const int64_t sms = sm_count();
+  auto rounds = [&](int64_t t) { return ceil_div(ceil_div(n, t) * ceil_div(p, t) * S, sms); };
+  const int64_t r64 = rounds(64);
+  const double t128 = 16384.0 * rounds(128), t64 = (vec ? 1.25 : 1.4) * 4096 * r64,
+               t32 = (vec ? 1.4 : 1.9) * 1024 * rounds(32);
+  if (!small_only && (t128 <= std::min(t64, t32) || ceil_div(n, 32) > 65535)) return 128;
+  return S <= kSimtCluster && r64 > 1 && t64 <= 1.03 * t32 ? 64 : 32;
+}
+
 }  // namespace
 
 SimtPlan simt_plan_for(bool f64, int64_t n, int64_t m, int64_t p, int sms) {
@@ -429,11 +653,11 @@ size_t simt_scratch_bytes(bool f64, int64_t n, int64_t m, int64_t p) {
 cudaError_t launch_simt_splitk_f32(int64_t n, int64_t m, int64_t p, const float *A, const float *B,
                                    float *C, float *part, const SimtPlan &pl, cudaStream_t s,
                                    const Epi *epi) {
-  if (pl.wide)
-    return launch_splitk<float, kSimtF32BM, kSimtF32BN, kSimtF32BK, 8, 8>(n, m, p, A, B, C, part, pl, s,
-                                                                         "simt_f32", nullptr, epi);
-  return launch_splitk<float, 64, 64, kSimtF32BK, 4, 4>(n, m, p, A, B, C, part, pl, s, "simt_f32",
-                                                        nullptr, epi);
+  const int tile = f32_tile(n, p, pl.S, f32_vec(A, B, C, m, p), !pl.wide || pl.S <= kSimtCluster);
+  if (tile == 32) return launch_ring<32, 32, 4>(n, m, p, A, B, C, part, pl.S, pl.ks, s, epi);
+  if (tile == 64) return launch_ring<64, 64, 8>(n, m, p, A, B, C, part, pl.S, pl.ks, s, epi);
+  return launch_splitk<float, kSimtF32BM, kSimtF32BN, kSimtF32BK, 8, 8>(n, m, p, A, B, C, part, pl, s,
+                                                                       "simt_f32", nullptr, epi);
 }
 
 // FP64 products whose 64 x 64 tiles leave the last round of the SMs partly empty
@@ -460,6 +684,9 @@ cudaError_t launch_simt_splitk_f64(int64_t n, int64_t m, int64_t p, const double
 
 cudaError_t launch_simt_f32(int64_t n, int64_t m, int64_t p, const float *A, const float *B,
                             float *C, cudaStream_t s, const Epi *epi) {
+  const int tile = f32_tile(n, p, 1, f32_vec(A, B, C, m, p), false);
+  if (tile == 32) return launch_ring<32, 32, 4>(n, m, p, A, B, C, nullptr, 1, m, s, epi);
+  if (tile == 64) return launch_ring<64, 64, 8>(n, m, p, A, B, C, nullptr, 1, m, s, epi);
   return launch_simt<float, kSimtF32BM, kSimtF32BN, kSimtF32BK, 8, 8>(n, m, p, A, B, C, s,
                                                                       "simt_f32", nullptr, epi);
 }
