@@ -180,6 +180,16 @@ size_t fp8_blocks_scratch_bytes(int64_t n, int64_t m, int64_t p);
 mm_status run_ozaki(Scratch &ws, int64_t n, int64_t m, int64_t p, const double *A,
                     const double *B, double *C, int S, bool gate, cudaStream_t s,
                     const Epi *epi = nullptr);
+// Several independent products, their level products in one launch.
+struct OzCall {
+  int64_t n, m, p;
+  const double *A, *B;
+  double *C;
+  int S;
+  bool gate;
+  const Epi *epi;
+};
+mm_status run_ozaki_many(Scratch &ws, const OzCall *calls, int count, cudaStream_t s);
 int64_t ozaki_chunk(int S);
 size_t ozaki_scratch_bytes(int64_t n, int64_t m, int64_t p, int S);
 // Grouped dispatch: split / SIMT / DGEMM tables in one launch per path.

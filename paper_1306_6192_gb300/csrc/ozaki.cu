@@ -85,6 +85,73 @@ constexpr int kRowChunk = 64;     // maxima: rows of B per strip item
 constexpr int kSeg = 16;          // digits: consecutive k per thread
 constexpr int kDigRows = 32;      // digits: rows of A (columns of B) per block
 
+// The kernels beside the level products take up to kOzItems products a launch, their
+// arguments in the launch's parameters: item g has the blocks from it[g].start.
+constexpr int kOzItems = 32;
+template <typename Item>
+struct OzItems {
+  int count;
+  Item it[kOzItems];
+};
+template <typename Item>
+__device__ __forceinline__ const Item &item_of(const OzItems<Item> &t, int block) {
+  int lo = 0, hi = t.count - 1;
+  while (lo < hi) {
+    const int mid = (lo + hi + 1) >> 1;
+    if (t.it[mid].start <= block) lo = mid;
+    else hi = mid - 1;
+  }
+  return t.it[lo];
+}
+// launch(items, blocks) over the items, kOzItems at a time; an item's start
+// holds its block count until then.
+template <typename Item, typename Launch>
+cudaError_t launch_items(const std::vector<Item> &items, Launch launch) {
+  for (size_t i = 0; i < items.size();) {
+    OzItems<Item> t{};
+    int64_t blocks = 0;
+    for (; i < items.size() && t.count < kOzItems; i++) {
+      const int64_t more = items[i].start;
+      if (blocks + more > 0x7fffffffLL) break;
+      Item &x = t.it[t.count++] = items[i];
+      x.start = (int32_t)blocks;
+      blocks += more;
+    }
+    const cudaError_t e = launch(t, (unsigned)blocks);
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
+}
+struct OzMaxItem {
+  const double *A, *B;
+  uint64_t *rowmax;  // n, then the column maxima
+  int64_t n, m, p;
+  int32_t start;
+};
+struct OzDigitItem {  // one K chunk [k0, k0 + mc)
+  const double *A, *B;
+  const uint64_t *rowmax;
+  int64_t n, m, p, k0, mc, a0, b0;
+  int32_t kt, bn, blocks_a, start;
+};
+struct OzSumItem {
+  const float *D;
+  const uint64_t *rowmax;
+  double *C;
+  const int *skip_if;
+  EpiT<double> epi;
+  int64_t plane, n, p;
+  int32_t chunks, gx, gy, start;
+};
+struct OzGateItem {
+  const float *G;
+  const uint64_t *rowmax;
+  int *flag;
+  int64_t plane, n, p;
+  float thr256;
+  int32_t chunks, gx, gy, start;
+};
+
 // Four consecutive doubles at a 32-byte boundary in one load.
 __device__ __forceinline__ void load4(const double *src, double (&v)[4]) {
   asm volatile("ld.global.v4.f64 {%0, %1, %2, %3}, [%4];"
@@ -248,26 +315,23 @@ __device__ __forceinline__ void emit_digits(int live, bool finite, int sigma, Ge
   if (GATE) put(S, make_uint4(gate[0], gate[1], gate[2], gate[3]));
 }
 
-// Maxima: items [0, ceil(n/8)) take 8 rows of A (a warp per row); the next ones
+// Maxima: blocks [0, ceil(n/8)) take 8 rows of A (a warp per row); the next ones
 // strips of 128 columns x 64 rows of B, merged into colmax with atomicMax on
-// the bit patterns (which order like the magnitudes); the rest write 256
-// entries each of the level launch's unit -> problem map (unit u belongs to
-// problem u / tiles).  Bound by reading A and B once: 32-byte loads where the
+// the bit patterns (which order like the magnitudes).
+// Bound by reading A and B once: 32-byte loads where the
 // rows allow them, eight in flight (268 MB at 4096^3 in 72 us).
 __global__ void __launch_bounds__(256)
-ozaki_max_kernel(const double *__restrict__ A, const double *__restrict__ B, int64_t n, int64_t m,
-                 int64_t p, uint64_t *__restrict__ rowmax, unsigned long long *__restrict__ colmax,
-                 int64_t max_items, int *__restrict__ map, int64_t units, int64_t tiles) {
+ozaki_max_kernel(const __grid_constant__ OzItems<OzMaxItem> items) {
   pdl_wait();
+  const OzMaxItem &it = item_of(items, blockIdx.x);
+  const double *__restrict__ A = it.A, *__restrict__ B = it.B;
+  uint64_t *rowmax = it.rowmax;
+  const int64_t n = it.n, m = it.m, p = it.p, block = (int)blockIdx.x - it.start;
+  unsigned long long *colmax = reinterpret_cast<unsigned long long *>(rowmax + n);
   const int64_t items_a = (n + kRowsPerItem - 1) / kRowsPerItem;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  if ((int64_t)blockIdx.x >= max_items) {
-    const int64_t u = ((int64_t)blockIdx.x - max_items) * 256 + threadIdx.x;
-    if (u < units) map[u] = (int)(u / tiles);
-    return;
-  }
-  if ((int64_t)blockIdx.x < items_a) {
-    const int64_t i = (int64_t)blockIdx.x * kRowsPerItem + warp;
+  if (block < items_a) {
+    const int64_t i = block * kRowsPerItem + warp;
     if (i >= n) return;
     const double *row = A + i * m;
     uint64_t mx = 0;
@@ -288,7 +352,7 @@ ozaki_max_kernel(const double *__restrict__ A, const double *__restrict__ B, int
     return;
   }
   __shared__ uint64_t part[8][kColStrip];
-  const int64_t b = (int64_t)blockIdx.x - items_a;
+  const int64_t b = block - items_a;
   const int64_t strips = (p + kColStrip - 1) / kColStrip;
   const int64_t c0 = (b % strips) * kColStrip, r0 = (b / strips) * kRowChunk;
   uint64_t mx[4] = {0, 0, 0, 0};
@@ -338,22 +402,25 @@ ozaki_max_kernel(const double *__restrict__ A, const double *__restrict__ B, int
 // with the accuracy gate's slice after them.
 //
 // Bound by instruction issue until the digits went in fp16 pairs (digit_pair;
-// through FP32 they cost 321 us at 4096^3 for 0.77 GB, now 197); blocks of a
+// through FP32 they cost 321 us at 4096^3 for 0.77 GB, now 165); blocks of a
 // quarter of a tile, since one of 256 columns by 128 k kept a small product's
 // few blocks busy for 100 us (192 served requests, 43 of them emulated: 12.0 ->
 // 8.9 ms).
 template <int S, bool GATE>
 __global__ void __launch_bounds__(256)
-ozaki_digits_kernel(const double *__restrict__ A, const double *__restrict__ B, int64_t n, int64_t m,
-                    int64_t p, int64_t k0, int64_t mc, int kt, int bn, unsigned blocks_a,
-                    const uint64_t *__restrict__ rowmax, const unsigned long long *__restrict__ colmax,
-                    uint4 *__restrict__ pack, int64_t a0, int64_t b0) {
+ozaki_digits_kernel(const __grid_constant__ OzItems<OzDigitItem> items, uint4 *__restrict__ pack) {
   constexpr int SS = S + (GATE ? 1 : 0);
   __shared__ double tile[128 * 32];
   pdl_wait();
+  const OzDigitItem &it = item_of(items, blockIdx.x);
+  const double *__restrict__ A = it.A, *__restrict__ B = it.B;
+  const uint64_t *__restrict__ rowmax = it.rowmax;
+  const int64_t n = it.n, m = it.m, p = it.p, k0 = it.k0, mc = it.mc, a0 = it.a0, b0 = it.b0;
+  const int kt = it.kt, bn = it.bn, block = (int)blockIdx.x - it.start;
+  const uint64_t *__restrict__ colmax = rowmax + n;
   const int tid = threadIdx.x, r = tid / 8, sg = tid % 8;
-  if (blockIdx.x < blocks_a) {
-    const int64_t o = blockIdx.x / kt, kb = blockIdx.x % kt;  // group of 32 rows, K block
+  if (block < it.blocks_a) {
+    const int64_t o = block / kt, kb = block % kt;  // group of 32 rows, K block
     const int64_t i = o * kDigRows + r;
     bool finite = true;
     const int sigma = i < n ? slice_exponent(rowmax[i], finite) : 0;
@@ -375,7 +442,7 @@ ozaki_digits_kernel(const double *__restrict__ A, const double *__restrict__ B, 
     });
     return;
   }
-  const unsigned b = blockIdx.x - blocks_a;
+  const int b = block - it.blocks_a;
   const int64_t o = b / kt, kb = b % kt;  // group of 32 columns, K block
   const int64_t c0 = o * kDigRows;
   double x[16];
@@ -430,17 +497,14 @@ __device__ __forceinline__ double int128_scaled(uint64_t lo, int64_t hi, int k) 
   return scalbn(d, k);
 }
 
-// The digit kernel of one K chunk, instantiated per S and gate (the slice loops
-// unroll with constant shifts).
-cudaError_t launch_ozaki_digits(int S, bool gate, int64_t blocks_a, int64_t blocks_b, cudaStream_t s,
-                                const double *A, const double *B, int64_t n, int64_t m,
-                                int64_t p, int64_t k0, int64_t mc, int kt, int bn,
-                                const uint64_t *rowmax, const unsigned long long *colmax,
-                                uint4 *pack, int64_t a0, int64_t b0) {
-  if (blocks_a + blocks_b > 0x7fffffffLL) return cudaErrorInvalidValue;
+// The digit kernel, instantiated per S and gate (the slice loops unroll with
+// constant shifts).
+cudaError_t launch_ozaki_digits(int S, bool gate, const std::vector<OzDigitItem> &items, uint4 *pack,
+                                cudaStream_t s) {
   auto launch = [&](auto kernel) {
-    return launch_pdl_if(blocks_a + blocks_b <= sm_count() * 4, kernel, (unsigned)(blocks_a + blocks_b), 256, 0,
-                         s, A, B, n, m, p, k0, mc, kt, bn, (unsigned)blocks_a, rowmax, colmax, pack, a0, b0);
+    return launch_items(items, [&](const OzItems<OzDigitItem> &t, unsigned blocks) {
+      return launch_pdl_if(blocks <= sm_count() * 4u, kernel, blocks, 256, 0, s, t, pack);
+    });
   };
   switch (S) {
 #define MM_OZ_DIG(V) \
@@ -484,8 +548,8 @@ __device__ __forceinline__ bool round_to_double(unsigned __int128 M, int k, uint
 // the level sums are integers below 2^24, so their weighted sum is formed
 // exactly in 128-bit integers and rounded once to FP64 (then scaled by a
 // power of two, which rounds again only in the subnormal range); NaN where
-// row i of A or column j of B is not finite.  A thread takes column j of the
-// rows blockIdx.y, blockIdx.y + gridDim.y, ...; the S level values of a chunk
+// row i of A or column j of B is not finite.  A thread takes column j of
+// every gy-th row; the S level values of a chunk
 // are loaded together, for V neighbouring columns at once (V = 2 halves the
 // loads where p is even; 211 -> 185 us at 4096^3).  One instantiation per S, so the level
 // loop unrolls without predicates.  The epilogue epi is applied to each entry; skip_if
@@ -493,11 +557,16 @@ __device__ __forceinline__ bool round_to_double(unsigned __int128 M, int k, uint
 // instead and this kernel writes nothing.
 template <int S, int V>
 __global__ void __launch_bounds__(256, V == 2 ? 3 : 4)
-ozaki_sum_kernel(const float *__restrict__ D, int64_t plane, int64_t n, int64_t p, int chunks,
-                 const uint64_t *__restrict__ rowmax, const unsigned long long *__restrict__ colmax,
-                 double *C, const int *skip_if, EpiT<double> epi) {
-  if (skip_if != nullptr && *reinterpret_cast<const volatile int *>(skip_if) != 0) return;
-  const int64_t j = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) * V;
+ozaki_sum_kernel(const __grid_constant__ OzItems<OzSumItem> items) {
+  const OzSumItem &it = item_of(items, blockIdx.x);
+  if (it.skip_if != nullptr && *reinterpret_cast<const volatile int *>(it.skip_if) != 0) return;
+  const float *__restrict__ D = it.D;
+  double *C = it.C;
+  const int64_t plane = it.plane, n = it.n, p = it.p;
+  const int chunks = it.chunks, block = (int)blockIdx.x - it.start, by = block / it.gx;
+  const uint64_t *__restrict__ rowmax = it.rowmax, *__restrict__ colmax = rowmax + n;
+  const EpiT<double> epi = it.epi;
+  const int64_t j = ((int64_t)(block % it.gx) * blockDim.x + threadIdx.x) * V;
   if (j >= p) return;
   bool fb[V];
   int tau[V];
@@ -508,7 +577,7 @@ ozaki_sum_kernel(const float *__restrict__ D, int64_t plane, int64_t n, int64_t 
   // at most kOzakiMaxChunks = 2^10 chunks), then v = X 32^(S-h) + Y once in
   // 128 bits
   constexpr int h = (S + 1) / 2;
-  for (int64_t i = blockIdx.y; i < n; i += gridDim.y) {
+  for (int64_t i = by; i < n; i += it.gy) {
     bool fa;
     const int sigma = slice_exponent(rowmax[i], fa);
     const int64_t x = i * p + j;
@@ -565,20 +634,16 @@ ozaki_sum_kernel(const float *__restrict__ D, int64_t plane, int64_t n, int64_t 
   }
 }
 
-// One wave of blocks (three or four a SM, the launch bounds); pairs of columns
-// where p is even and wide enough to fill the blocks.
-cudaError_t launch_ozaki_sum(int S, cudaStream_t s, const float *D, int64_t plane, int64_t n, int64_t p,
-                             int chunks, const uint64_t *rowmax, const unsigned long long *colmax,
-                             double *C, const int *skip_if, const EpiT<double> &epi) {
-  const int v = (p & 1) == 0 && p >= 512 ? 2 : 1;
-  const int64_t gx = ceil_div(p, 256 * v);
-  const int64_t gy = std::max<int64_t>(
-      1, std::min<int64_t>({n, 65535, ceil_div((int64_t)sm_count() * (v == 2 ? 3 : 4), gx)}));
-  if (gx > 0x7fffffffLL) return cudaErrorInvalidValue;
+// Pairs of columns where p is even and wide enough to fill the blocks.
+int sum_columns(int64_t p) { return (p & 1) == 0 && p >= 512 ? 2 : 1; }
+
+// The sum kernel over products of one S and one V = sum_columns.
+cudaError_t launch_ozaki_sum(int S, int v, const std::vector<OzSumItem> &items, cudaStream_t s) {
   auto launch = [&](auto kernel) {
-    kernel<<<dim3((unsigned)gx, (unsigned)gy), 256, 0, s>>>(D, plane, n, p, chunks, rowmax, colmax, C,
-                                                            skip_if, epi);
-    return cudaGetLastError();
+    return launch_items(items, [&](const OzItems<OzSumItem> &t, unsigned blocks) {
+      kernel<<<blocks, 256, 0, s>>>(t);
+      return cudaGetLastError();
+    });
   };
   switch (S) {
 #define MM_OZ_SUM(W) \
@@ -588,6 +653,21 @@ cudaError_t launch_ozaki_sum(int S, cudaStream_t s, const float *D, int64_t plan
 #undef MM_OZ_SUM
     default: return cudaErrorInvalidValue;
   }
+}
+
+// Blocks of a product in a kernel whose blocks take gx column groups and, each,
+// every gy-th row: a wave of `per_sm` a SM, or, among other products, at least
+// eight rows a block.
+template <typename Item>
+bool row_blocks(Item &it, int64_t columns, int per_sm, bool alone) {
+  const int64_t gx = ceil_div(it.p, columns);
+  const int64_t rows = alone ? it.n : ceil_div(it.n, 8);
+  const int64_t gy = std::max<int64_t>(1, std::min<int64_t>({rows, 65535, ceil_div((int64_t)sm_count() * per_sm, gx)}));
+  if (gx * gy > 0x7fffffffLL) return false;
+  it.gx = (int32_t)gx;
+  it.gy = (int32_t)gy;
+  it.start = (int32_t)(gx * gy);
+  return true;
 }
 
 // Accuracy gate.  Every term a_ir b_rj of the emulated product is off by at
@@ -608,15 +688,19 @@ cudaError_t launch_ozaki_sum(int S, cudaStream_t s, const float *D, int64_t plan
 // terms), lowers the sum by 2^-10 (more than that addition's rounding) and
 // sets a flag where any entry with a finite, non-zero row and column misses
 // the threshold; the FP64 FMA product then recomputes C.
-// A block takes 1024 columns of the rows blockIdx.y, + gridDim.y, ...; a thread
+// A block takes 1024 columns of every gy-th row; a thread
 // columns 256 apart, whose maxima it reads once.
 // (43 -> 20 us at 4096^3 against a row per block and a column per thread and turn.)
 constexpr int kGateCols = 4;
 __global__ void __launch_bounds__(256)
-ozaki_gate_check_kernel(const float *__restrict__ G, int64_t plane, int chunks, int64_t n,
-                        int64_t p, const uint64_t *__restrict__ rowmax,
-                        const unsigned long long *__restrict__ colmax, float thr256, int *flag) {
-  const int64_t j0 = (int64_t)blockIdx.x * (256 * kGateCols) + threadIdx.x;
+ozaki_gate_check_kernel(const __grid_constant__ OzItems<OzGateItem> items) {
+  const OzGateItem &it = item_of(items, blockIdx.x);
+  const float *__restrict__ G = it.G;
+  const int64_t plane = it.plane, n = it.n, p = it.p;
+  const int chunks = it.chunks, block = (int)blockIdx.x - it.start, by = block / it.gx;
+  const uint64_t *__restrict__ rowmax = it.rowmax, *__restrict__ colmax = rowmax + n;
+  const float thr256 = it.thr256;
+  const int64_t j0 = (int64_t)(block % it.gx) * (256 * kGateCols) + threadIdx.x;
   bool live[kGateCols];
 #pragma unroll
   for (int q = 0; q < kGateCols; q++) {
@@ -627,7 +711,7 @@ ozaki_gate_check_kernel(const float *__restrict__ G, int64_t plane, int chunks, 
   }
   bool fail = false;
 #pragma unroll 2
-  for (int64_t i = blockIdx.y; i < n; i += gridDim.y) {
+  for (int64_t i = by; i < n; i += it.gy) {
     bool fi;
     slice_exponent(rowmax[i], fi);
     // a row with a NaN or an infinity gives NaN by design; an all-zero row
@@ -644,17 +728,16 @@ ozaki_gate_check_kernel(const float *__restrict__ G, int64_t plane, int chunks, 
 #pragma unroll
     for (int q = 0; q < kGateCols; q++) fail |= !(v[q] * (1.0f - 0x1p-10f) >= thr256);
   }
-  if (__syncthreads_or(fail) && threadIdx.x == 0) atomicOr(flag, 1);
+  if (__syncthreads_or(fail) && threadIdx.x == 0) atomicOr(it.flag, 1);
 }
 
-// Scratch offsets of one call.
+// Scratch offsets of one product (pack rows and bytes from the scratch's start).
 struct OzLayout {
   int S, SS, chunks, bn, mt, nt;
-  int64_t mc;
+  int64_t mc, tiles;
   std::vector<int64_t> k0, kc, kt, a0, b0;
-  int64_t rows = 0, plane = 0;
-  size_t max_off, zero_off, flag_off, zero_end, d_off, tab_off, map_off, simt_off, need;
-  int64_t units = 0;
+  int64_t plane = 0;
+  size_t max_off, flag_off, d_off;
 };
 
 }  // namespace
@@ -664,194 +747,279 @@ int64_t ozaki_chunk(int S) {
   return mc;
 }
 
-mm_status run_ozaki(Scratch &ws, int64_t n, int64_t m, int64_t p, const double *A,
-                    const double *B, double *C, int S, bool gate, cudaStream_t s, const Epi *epi) {
+// Lays one product out behind `rows` pack rows and appends its level and gate
+// problems to the table (C: the plane's index; unit_start unset).
+static mm_status ozaki_layout(const OzCall &q, int64_t &rows, OzLayout &lay, TcChoice &ch,
+                              std::vector<SplitProb> &tab) {
+  const int S = q.S;
   if (S < kOzakiMinSlices || S > kOzakiMaxSlices) return MM_EINVAL;
-  if (n == 0 || p == 0) return MM_OK;
-  if (m == 0) return note_cuda(cudaMemsetAsync(C, 0, (size_t)(n * p) * sizeof(double), s));
-  OzLayout lay;
   lay.S = S;
-  lay.SS = S + (gate ? 1 : 0);  // slices per tile in the packs (the gate's last)
+  lay.SS = S + (q.gate ? 1 : 0);  // slices per tile in the packs (the gate's last)
   lay.mc = ozaki_chunk(S);
-  if (ceil_div(m, lay.mc) > kOzakiMaxChunks) return MM_EINVAL;
-  lay.chunks = (int)ceil_div(m, lay.mc);
-  TcChoice ch = tune_choose(n, std::min(m, lay.mc), p);
+  if (ceil_div(q.m, lay.mc) > kOzakiMaxChunks) return MM_EINVAL;
+  lay.chunks = (int)ceil_div(q.m, lay.mc);
+  ch = tune_choose(q.n, std::min(q.m, lay.mc), q.p);
   lay.bn = tc_bn(kTcE4m3, ch.bn);
-  lay.mt = (int)ceil_div(n, kTcBM);
-  lay.nt = (int)ceil_div(p, lay.bn);
+  lay.mt = (int)ceil_div(q.n, kTcBM);
+  lay.nt = (int)ceil_div(q.p, lay.bn);
   for (int c = 0; c < lay.chunks; c++) {
-    const int64_t k0 = (int64_t)c * lay.mc, kc = std::min(lay.mc, m - k0);
+    const int64_t k0 = (int64_t)c * lay.mc, kc = std::min(lay.mc, q.m - k0);
     const int64_t kt = ceil_div(kc, 128);
     lay.k0.push_back(k0);
     lay.kc.push_back(kc);
     lay.kt.push_back(kt);
-    lay.a0.push_back(lay.rows);
-    lay.rows += (int64_t)lay.mt * lay.SS * kt * kTcBM;
-    lay.b0.push_back(lay.rows);
-    lay.rows += (int64_t)lay.nt * lay.SS * kt * lay.bn;
+    lay.a0.push_back(rows);
+    rows += (int64_t)lay.mt * lay.SS * kt * kTcBM;
+    lay.b0.push_back(rows);
+    rows += (int64_t)lay.nt * lay.SS * kt * lay.bn;
   }
-  if (lay.rows > 0x7fffffffLL) return MM_EINVAL;
-  // S level problems per chunk, then the gate's product per chunk
-  const int nprobs = lay.chunks * lay.SS;
-  const int64_t tiles = (int64_t)lay.mt * lay.nt;
+  if (rows > 0x7fffffffLL) return MM_EINVAL;
+  lay.tiles = (int64_t)lay.mt * lay.nt;
   // level planes of D, padded so that the planes of one entry do not sit a
   // power of two apart (128-byte aligned)
-  lay.plane = (n * p + 31) / 32 * 32 + 32;
-  std::vector<SplitProb> tab((size_t)nprobs);
+  lay.plane = (q.n * q.p + 31) / 32 * 32 + 32;
   // level problems, longest K first (the persistent grid takes units in
-  // order, so the short ones fill the last wave); problem g = (S-1-L) *
-  // chunks + c holds units [g T, (g+1) T) of the T tiles.  (Interleaving the
+  // order, so the short ones fill the last wave).  (Interleaving the
   // levels tile by tile was measured slower: 19 GB of DRAM reads per 4096^3
-  // launch instead of 11, 5.4 ms instead of 4.6.)
-  int g = 0;
-  for (int L = S - 1; L >= 0; L--)
-    for (int c = 0; c < lay.chunks; c++, g++) {
-      SplitProb &sp = tab[(size_t)g];
-      std::memset(&sp, 0, sizeof(sp));
-      const int64_t kt = lay.kt[(size_t)c];
-      sp.n = (int32_t)n;
-      sp.p = (int32_t)p;
-      sp.kt = (int32_t)((L + 1) * kt);
-      sp.m = sp.kt * 128;  // padded K of the level: zero digits past the chunk
-      sp.mt = lay.mt;
-      sp.nt = lay.nt;
-      sp.bn = lay.bn;
-      sp.group_m = ch.group_m;
-      sp.a_row0 = lay.a0[(size_t)c];
-      sp.b_row0 = lay.b0[(size_t)c] + (int64_t)(S - 1 - L) * kt * lay.bn;
-      sp.a_kstride = (int32_t)(lay.SS * kt);
-      sp.b_kstride = (int32_t)(lay.SS * kt);
-      sp.unit_start = (int32_t)lay.units;
-      lay.units += tiles;
-      sp.split_from = (int32_t)tiles;
-      sp.split_s = 1;
-      sp.C = reinterpret_cast<float *>((uintptr_t)(((int64_t)c * S + L) * lay.plane));  // offset
-    }
-  // the gate's products (one slice against one slice: as short as level 0,
-  // so they run last), planes after the level planes
-  for (int c = 0; gate && c < lay.chunks; c++, g++) {
-    SplitProb &sp = tab[(size_t)g];
+  // launch instead of 11, 5.4 ms instead of 4.6.)  The gate's products (one
+  // slice against one slice: as short as level 0) come last, planes after the
+  // level planes.
+  auto add = [&](int c, int64_t levels, int64_t a_slice, int64_t b_slice, int64_t plane) {
+    SplitProb sp;
     std::memset(&sp, 0, sizeof(sp));
     const int64_t kt = lay.kt[(size_t)c];
-    sp.n = (int32_t)n;
-    sp.p = (int32_t)p;
-    sp.kt = (int32_t)kt;
-    sp.m = sp.kt * 128;
+    sp.n = (int32_t)q.n;
+    sp.p = (int32_t)q.p;
+    sp.kt = (int32_t)(levels * kt);
+    sp.m = sp.kt * 128;  // padded K of the level: zero digits past the chunk
     sp.mt = lay.mt;
     sp.nt = lay.nt;
     sp.bn = lay.bn;
     sp.group_m = ch.group_m;
-    sp.a_row0 = lay.a0[(size_t)c] + (int64_t)S * kt * kTcBM;
-    sp.b_row0 = lay.b0[(size_t)c] + (int64_t)S * kt * lay.bn;
+    sp.a_row0 = lay.a0[(size_t)c] + a_slice * kt * kTcBM;
+    sp.b_row0 = lay.b0[(size_t)c] + b_slice * kt * lay.bn;
     sp.a_kstride = (int32_t)(lay.SS * kt);
     sp.b_kstride = (int32_t)(lay.SS * kt);
-    sp.unit_start = (int32_t)lay.units;
-    lay.units += tiles;
-    sp.split_from = (int32_t)tiles;
+    sp.split_from = (int32_t)lay.tiles;
     sp.split_s = 1;
-    sp.C = reinterpret_cast<float *>((uintptr_t)(((int64_t)lay.chunks * S + c) * lay.plane));
-  }
-  if (lay.units > 0x7fffffffLL) return MM_EINVAL;
-  const size_t pack_bytes = (size_t)lay.rows * kPackRowBytes;
-  lay.max_off = (pack_bytes + 255) & ~(size_t)255;  // row maxima (n) + column maxima (p)
-  lay.zero_off = lay.max_off;
-  // + zero scale words, the gate's fallback flag
-  lay.flag_off = lay.max_off + (size_t)(n + p) * 8 + (size_t)(n + p) * 4;
-  lay.zero_end = lay.flag_off + sizeof(int);
-  lay.d_off = (lay.zero_end + 255) & ~(size_t)255;
-  lay.tab_off = (lay.d_off + (size_t)nprobs * lay.plane * sizeof(float) + 255) & ~(size_t)255;
-  // the table, then the work units of each CTA (the levels differ in length)
-  TcConfig cfg{128, 4, ch.grid};
-  cfg.max_bn = lay.bn;
-  std::vector<int> order;
-  tc_unit_order(tab.data(), nprobs, tc_launch_grid(cfg, lay.units), order);
-  const size_t tab_bytes = ((size_t)nprobs * sizeof(SplitProb) + 15) & ~(size_t)15;
-  lay.map_off = (lay.tab_off + tab_bytes + order.size() * sizeof(int) + 255) & ~(size_t)255;
-  // the fallback's K-slice partials (under-filled products)
-  lay.simt_off = (lay.map_off + (size_t)lay.units * sizeof(int) + 255) & ~(size_t)255;
-  lay.need = lay.simt_off + simt_scratch_bytes(true, n, m, p);
-  cudaError_t e = ws.reserve(lay.need, s);
-  if (e != cudaSuccess) return note_cuda(e);
-  uint8_t *base = static_cast<uint8_t *>(ws.ptr);
-  uint64_t *rowmax = reinterpret_cast<uint64_t *>(base + lay.max_off);
-  unsigned long long *colmax = reinterpret_cast<unsigned long long *>(rowmax + n);
-  uint32_t *zero_words = reinterpret_cast<uint32_t *>(colmax + p);
-  float *D = reinterpret_cast<float *>(base + lay.d_off);
-  for (auto &sp : tab) {
-    sp.C = D + (uintptr_t)sp.C;
-    sp.sA = zero_words;      // scale exponent 0: the digits are not rescaled
-    sp.tB = zero_words + n;
-  }
-  SplitProb *d_tab = reinterpret_cast<SplitProb *>(base + lay.tab_off);
-  const int *d_order = reinterpret_cast<const int *>(base + lay.tab_off + tab_bytes);
-  {
-    std::vector<uint8_t> blob(tab_bytes + order.size() * sizeof(int), 0);
-    std::memcpy(blob.data(), tab.data(), tab.size() * sizeof(SplitProb));
-    std::memcpy(blob.data() + tab_bytes, order.data(), order.size() * sizeof(int));
-    e = ws.stage.copy_to_device(d_tab, blob.data(), blob.size(), s);
-  }
-  if (e == cudaSuccess) e = cudaMemsetAsync(base + lay.zero_off, 0, lay.zero_end - lay.zero_off, s);
-  if (e != cudaSuccess) return note_cuda(e);
-  int *unit_map = reinterpret_cast<int *>(base + lay.map_off);
-  {
-    TraceScope ts("ozaki_max", s);
-    const int64_t items = ceil_div(n, kRowsPerItem) + ceil_div(p, kColStrip) * ceil_div(m, kRowChunk);
-    const int64_t blocks = items + ceil_div(lay.units, 256);
-    if (blocks > 0x7fffffffLL) return MM_EINVAL;
-    e = launch_pdl_if(blocks <= sm_count() * 4, ozaki_max_kernel, (unsigned)blocks, 256, 0, s, A, B, n, m, p,
-                      rowmax, colmax, items, unit_map, lay.units, tiles);
+    sp.C = reinterpret_cast<float *>((uintptr_t)(plane * lay.plane));  // offset
+    tab.push_back(sp);
+  };
+  for (int L = S - 1; L >= 0; L--)
+    for (int c = 0; c < lay.chunks; c++) add(c, L + 1, 0, S - 1 - L, (int64_t)c * S + L);
+  for (int c = 0; q.gate && c < lay.chunks; c++) add(c, 1, S, S, (int64_t)lay.chunks * S + c);
+  return MM_OK;
+}
+
+mm_status run_ozaki(Scratch &ws, int64_t n, int64_t m, int64_t p, const double *A,
+                    const double *B, double *C, int S, bool gate, cudaStream_t s, const Epi *epi) {
+  const OzCall q{n, m, p, A, B, C, S, gate, epi};
+  return run_ozaki_many(ws, &q, 1, s);
+}
+
+mm_status run_ozaki_many(Scratch &ws, const OzCall *calls, int count, cudaStream_t s) {
+  std::vector<OzCall> qs;
+  for (int g = 0; g < count; g++) {
+    const OzCall &q = calls[g];
+    if (q.S < kOzakiMinSlices || q.S > kOzakiMaxSlices) return MM_EINVAL;
+    if (q.n == 0 || q.p == 0) continue;
+    if (q.m > 0) {
+      qs.push_back(q);
+      continue;
+    }
+    const cudaError_t e = cudaMemsetAsync(q.C, 0, (size_t)(q.n * q.p) * sizeof(double), s);
     if (e != cudaSuccess) return note_cuda(e);
   }
+  if (qs.empty()) return MM_OK;
+  const size_t nq = qs.size();
+  std::vector<OzLayout> lays(nq);
+  std::vector<SplitProb> tab;
+  std::vector<int> owner;  // problem -> product
+  TcConfig cfg{128, 4, 0};
+  int64_t rows = 0;
+  for (size_t g = 0; g < nq; g++) {
+    TcChoice ch;
+    const mm_status st = ozaki_layout(qs[g], rows, lays[g], ch, tab);
+    if (st != MM_OK) return st;
+    owner.resize(tab.size(), (int)g);
+    cfg.max_bn = std::max(cfg.max_bn, lays[g].bn);
+    if (nq == 1) cfg.grid = ch.grid;
+  }
+  auto align256 = [](size_t x) { return (x + 255) & ~(size_t)255; };
+  // row maxima (n) + column maxima (p), zero scale words and the gate's fallback
+  // flag of each product, then the planes
+  size_t off = align256((size_t)rows * kPackRowBytes), simt_bytes = 0;
+  const size_t zero_off = off;
+  for (size_t g = 0; g < nq; g++) {
+    const OzCall &q = qs[g];
+    lays[g].max_off = off;
+    lays[g].flag_off = off + (size_t)(q.n + q.p) * 12;
+    off = (lays[g].flag_off + sizeof(int) + 7) & ~(size_t)7;
+    simt_bytes = std::max(simt_bytes, simt_scratch_bytes(true, q.n, q.m, q.p));
+  }
+  const size_t zero_end = off;
+  for (size_t g = 0; g < nq; g++) {
+    lays[g].d_off = align256(off);
+    off = lays[g].d_off + (size_t)lays[g].chunks * lays[g].SS * lays[g].plane * sizeof(float);
+  }
+  const size_t tab_off = align256(off);
+  const int nprobs = (int)tab.size();
+  // several products in one launch: longest units first over all of them
+  std::vector<int> by_length((size_t)nprobs);
+  for (int g = 0; g < nprobs; g++) by_length[(size_t)g] = g;
+  if (nq > 1)
+    std::stable_sort(by_length.begin(), by_length.end(), [&](int a, int b) {
+      return (int64_t)tab[(size_t)a].kt * tab[(size_t)a].bn > (int64_t)tab[(size_t)b].kt * tab[(size_t)b].bn;
+    });
+  int64_t units = 0;
+  std::vector<SplitProb> sorted;
+  std::vector<int> map;  // unit -> problem
+  for (int g : by_length) {
+    SplitProb sp = tab[(size_t)g];
+    const int64_t tiles = lays[(size_t)owner[(size_t)g]].tiles;
+    if (units + tiles > 0x7fffffffLL) return MM_EINVAL;
+    sp.unit_start = (int32_t)units;
+    map.insert(map.end(), (size_t)tiles, (int)sorted.size());
+    units += tiles;
+    sorted.push_back(sp);
+  }
+  // the table, then the work units of each CTA (the levels differ in length), the
+  // unit map
+  const int grid = tc_launch_grid(cfg, units);
+  const size_t tab_bytes = ((size_t)nprobs * sizeof(SplitProb) + 15) & ~(size_t)15;
+  const size_t order_end = (tab_bytes + ((size_t)grid + 1 + (size_t)units) * sizeof(int) + 255) & ~(size_t)255;
+  const size_t map_off = tab_off + order_end;
+  // the fallbacks' K-slice partials (under-filled products)
+  const size_t simt_off = align256(map_off + (size_t)units * sizeof(int));
+  cudaError_t e = ws.reserve(simt_off + simt_bytes, s);
+  if (e != cudaSuccess) return note_cuda(e);
+  uint8_t *base = static_cast<uint8_t *>(ws.ptr);
+  for (int k = 0; k < nprobs; k++) {
+    const size_t g = (size_t)owner[(size_t)by_length[(size_t)k]];
+    SplitProb &sp = sorted[(size_t)k];
+    sp.C = reinterpret_cast<float *>(base + lays[g].d_off) + (uintptr_t)sp.C;
+    // scale exponent 0: the digits are not rescaled
+    sp.sA = reinterpret_cast<uint32_t *>(base + lays[g].max_off + (size_t)(qs[g].n + qs[g].p) * 8);
+    sp.tB = sp.sA + qs[g].n;
+  }
+  SplitProb *d_tab = reinterpret_cast<SplitProb *>(base + tab_off);
+  const int *d_order = reinterpret_cast<const int *>(base + tab_off + tab_bytes);
+  int *unit_map = reinterpret_cast<int *>(base + map_off);
+  e = cudaMemsetAsync(base + zero_off, 0, zero_end - zero_off, s);
+  if (e != cudaSuccess) return note_cuda(e);
+  auto rowmax = [&](size_t g) { return reinterpret_cast<uint64_t *>(base + lays[g].max_off); };
+  auto planes = [&](size_t g) { return reinterpret_cast<const float *>(base + lays[g].d_off); };
+  auto flag = [&](size_t g) { return reinterpret_cast<int *>(base + lays[g].flag_off); };
   {
-    TraceScope ts("ozaki_digits", s);
-    uint4 *pk = static_cast<uint4 *>(ws.ptr);
-    for (int c = 0; c < lay.chunks; c++) {
-      const int kt = (int)lay.kt[(size_t)c];
-      e = launch_ozaki_digits(S, gate, (int64_t)lay.mt * (kTcBM / kDigRows) * kt,
-                              (int64_t)lay.nt * (lay.bn / kDigRows) * kt, s, A, B, n, m, p,
-                              lay.k0[(size_t)c], lay.kc[(size_t)c], kt, lay.bn, rowmax, colmax, pk,
-                              lay.a0[(size_t)c], lay.b0[(size_t)c]);
+    TraceScope ts("ozaki_max", s);
+    std::vector<OzMaxItem> items;
+    for (size_t g = 0; g < nq; g++) {
+      const OzCall &q = qs[g];
+      const int64_t blocks = ceil_div(q.n, kRowsPerItem) + ceil_div(q.p, kColStrip) * ceil_div(q.m, kRowChunk);
+      if (blocks > 0x7fffffffLL) return MM_EINVAL;
+      items.push_back({q.A, q.B, rowmax(g), q.n, q.m, q.p, (int32_t)blocks});
+    }
+    e = launch_items(items, [&](const OzItems<OzMaxItem> &t, unsigned blocks) {
+      return launch_pdl_if(blocks <= sm_count() * 4u, ozaki_max_kernel, blocks, 256, 0, s, t);
+    });
+    if (e != cudaSuccess) return note_cuda(e);
+  }
+  // products of one slice count (gate, column pairing) share a launch
+  for (int S = kOzakiMinSlices; S <= kOzakiMaxSlices; S++)
+    for (int gate = 0; gate < 2; gate++) {
+      std::vector<OzDigitItem> items;
+      for (size_t g = 0; g < nq; g++) {
+        const OzCall &q = qs[g];
+        const OzLayout &lay = lays[g];
+        if (q.S != S || q.gate != (gate != 0)) continue;
+        for (size_t c = 0; c < (size_t)lay.chunks; c++) {
+          const int64_t blocks_a = (int64_t)lay.mt * (kTcBM / kDigRows) * lay.kt[c];
+          const int64_t blocks = blocks_a + (int64_t)lay.nt * (lay.bn / kDigRows) * lay.kt[c];
+          if (blocks > 0x7fffffffLL) return MM_EINVAL;
+          items.push_back({q.A, q.B, rowmax(g), q.n, q.m, q.p, lay.k0[c], lay.kc[c], lay.a0[c], lay.b0[c],
+                           (int32_t)lay.kt[c], lay.bn, (int32_t)blocks_a, (int32_t)blocks});
+        }
+      }
+      if (items.empty()) continue;
+      TraceScope ts("ozaki_digits", s);
+      e = launch_ozaki_digits(S, gate != 0, items, static_cast<uint4 *>(ws.ptr), s);
       if (e != cudaSuccess) return note_cuda(e);
     }
+  // while the digits are made: the units' order (alone 0.2 ms at 4096^3)
+  {
+    std::vector<int> order;
+    tc_unit_order(sorted.data(), nprobs, grid, order);
+    std::vector<uint8_t> blob(order_end + map.size() * sizeof(int), 0);
+    std::memcpy(blob.data(), sorted.data(), sorted.size() * sizeof(SplitProb));
+    std::memcpy(blob.data() + tab_bytes, order.data(), order.size() * sizeof(int));
+    std::memcpy(blob.data() + order_end, map.data(), map.size() * sizeof(int));
+    e = ws.stage.copy_to_device(d_tab, blob.data(), blob.size(), s);
+    if (e != cudaSuccess) return note_cuda(e);
   }
-  e = launch_tc(kTcE4m3, device_table(d_tab, nprobs), (int)lay.units, unit_map, nullptr, ws.ptr, lay.rows, cfg,
+  e = launch_tc(kTcE4m3, device_table(d_tab, nprobs), (int)units, unit_map, nullptr, ws.ptr, rows, cfg,
                 g_ctx.d_err, s, d_order);
   if (e != cudaSuccess) return note_cuda(e);
   // the gate reads the level sums only, so it runs before the sum kernel:
   // where it fails, the sum writes nothing and the FP64 FMA product below
   // reads the epilogue's D (which may be C) untouched
-  int *flag = gate ? reinterpret_cast<int *>(base + lay.flag_off) : nullptr;
-  if (gate) {
-    TraceScope ts("ozaki_gate", s);
-    const double room = 0.98 - (double)m * 0x1p-23;
+  std::vector<OzGateItem> gates;
+  for (size_t g = 0; g < nq; g++) {
+    const OzCall &q = qs[g];
+    const OzLayout &lay = lays[g];
+    if (!q.gate) continue;
+    const double room = 0.98 - (double)q.m * 0x1p-23;
     const double thr256 = room < 0.5 ? (double)INFINITY
-                                     : 256.0 * std::sqrt((double)m) * (S + 2) *
-                                           std::ldexp(1.0, -5 * S - 1) * 1e14 / room;
+                                     : 256.0 * std::sqrt((double)q.m) * (q.S + 2) *
+                                           std::ldexp(1.0, -5 * q.S - 1) * 1e14 / room;
     float thr = (float)thr256;  // rounded up to a float
     if ((double)thr < thr256) thr = std::nextafter(thr, (float)INFINITY);
-    const int64_t gx = ceil_div(p, 256 * kGateCols);
-    const int64_t gy = std::max<int64_t>(1, std::min<int64_t>({n, 65535, ceil_div((int64_t)sm_count() * 8, gx)}));
-    if (gx > 0x7fffffffLL) return MM_EINVAL;
+    OzGateItem it{planes(g) + (int64_t)lay.chunks * q.S * lay.plane, rowmax(g), flag(g), lay.plane, q.n, q.p, thr,
+                  lay.chunks, 0, 0, 0};
+    if (!row_blocks(it, 256 * kGateCols, 8, nq == 1)) return MM_EINVAL;
+    gates.push_back(it);
+  }
+  if (!gates.empty()) {
+    TraceScope ts("ozaki_gate", s);
     // (not as a dependent: its blocks would wait beside the level products for
     // all of their time)
-    ozaki_gate_check_kernel<<<dim3((unsigned)gx, (unsigned)gy), 256, 0, s>>>(
-        D + (int64_t)lay.chunks * S * lay.plane, lay.plane, lay.chunks, n, p, rowmax, colmax, thr, flag);
-    if ((e = cudaGetLastError()) != cudaSuccess) return note_cuda(e);
-  }
-  {
-    TraceScope ts("ozaki_sum", s);
-    e = launch_ozaki_sum(S, s, D, lay.plane, n, p, lay.chunks, rowmax, colmax, C, flag, epi_of<double>(epi));
+    e = launch_items(gates, [&](const OzItems<OzGateItem> &t, unsigned blocks) {
+      ozaki_gate_check_kernel<<<blocks, 256, 0, s>>>(t);
+      return cudaGetLastError();
+    });
     if (e != cudaSuccess) return note_cuda(e);
   }
-  if (!gate) return MM_OK;
+  for (int S = kOzakiMinSlices; S <= kOzakiMaxSlices; S++)
+    for (int v = 1; v <= 2; v++) {
+      std::vector<OzSumItem> items;
+      for (size_t g = 0; g < nq; g++) {
+        const OzCall &q = qs[g];
+        if (q.S != S || sum_columns(q.p) != v) continue;
+        OzSumItem it{planes(g), rowmax(g), q.C, q.gate ? flag(g) : nullptr, epi_of<double>(q.epi),
+                     lays[g].plane, q.n, q.p, lays[g].chunks, 0, 0, 0};
+        // one wave of blocks: three or four a SM, the launch bounds
+        if (!row_blocks(it, 256 * v, v == 2 ? 3 : 4, nq == 1)) return MM_EINVAL;
+        items.push_back(it);
+      }
+      if (items.empty()) continue;
+      TraceScope ts("ozaki_sum", s);
+      e = launch_ozaki_sum(S, v, items, s);
+      if (e != cudaSuccess) return note_cuda(e);
+    }
   // the FP64 FMA product replaces C where the flag is set: the same kernels
   // and K slices as MM_MODE_DGEMM, so the bits are that mode's
-  const SimtPlan pl = simt_plan(true, n, m, p);
-  if (pl.S >= 1)
-    return note_cuda(launch_simt_splitk_f64(
-        n, m, p, A, B, C, pl.S > 1 ? reinterpret_cast<double *>(base + lay.simt_off) : nullptr, pl, s,
-        flag, epi));
-  return note_cuda(launch_simt_f64(n, m, p, A, B, C, s, flag, epi));
+  for (size_t g = 0; g < nq; g++) {
+    const OzCall &q = qs[g];
+    if (!q.gate) continue;
+    const SimtPlan pl = simt_plan(true, q.n, q.m, q.p);
+    if (pl.S >= 1)
+      e = launch_simt_splitk_f64(q.n, q.m, q.p, q.A, q.B, q.C,
+                                 pl.S > 1 ? reinterpret_cast<double *>(base + simt_off) : nullptr, pl, s, flag(g),
+                                 q.epi);
+    else
+      e = launch_simt_f64(q.n, q.m, q.p, q.A, q.B, q.C, s, flag(g), q.epi);
+    if (e != cudaSuccess) return note_cuda(e);
+  }
+  return MM_OK;
 }
 
 size_t ozaki_scratch_bytes(int64_t n, int64_t m, int64_t p, int S) {

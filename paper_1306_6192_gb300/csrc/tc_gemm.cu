@@ -673,7 +673,11 @@ int tc_launch_grid(const TcConfig &cfg, int64_t total_units) {
 
 void tc_unit_order(const SplitProb *tab, int nprobs, int grid, std::vector<int> &out) {
   int64_t total = 0;
-  for (int g = 0; g < nprobs; g++) total += split_units(tab[g]);
+  int max_bn = 1;
+  for (int g = 0; g < nprobs; g++) {
+    total += split_units(tab[g]);
+    max_bn = std::max(max_bn, (int)tab[g].bn);
+  }
   out.assign((size_t)grid + 1 + (size_t)total, 0);
   if (grid <= 0) return;
   // (expected free time, CTA): a binary heap on the earliest time, lowest CTA
@@ -699,7 +703,7 @@ void tc_unit_order(const SplitProb *tab, int nprobs, int grid, std::vector<int> 
       auto &slot = heap.back();
       owner[(size_t)(pr.unit_start + t)] = slot.second;
       count[(size_t)slot.second]++;
-      slot.first += rows + 1;
+      slot.first += (rows * pr.bn + max_bn - 1) / max_bn + 1;  // narrower tiles take less
       std::push_heap(heap.begin(), heap.end(), later);
     }
   }
