@@ -123,9 +123,6 @@ struct SplitProb {
   // kt, the layout above); a larger stride lets a product read a window of
   // kt K blocks out of a longer pack (the FP64 emulation's level products)
   int32_t a_kstride, b_kstride;
-  // 1 + index of C's tensor map in the launch's map array (tiled stores of
-  // the epilogue); 0: C is written with plain stores
-  int32_t c_tma;
   // kTcSplitF16x3: the product's state words (HalfState) on the device
   int32_t *hx;
   // K blocks that it sums in one accumulator (a power of two)
@@ -296,7 +293,7 @@ cudaError_t launch_tc(TcKind kind, const ProbTable &tab, int total_units, const 
                       const int *flags,
                       void *pack_base, int64_t pack_rows, const TcConfig &cfg,
                       int *d_err, cudaStream_t s, const int *order = nullptr,
-                      int uniform_only = 0, const void *c_maps = nullptr, int *clear = nullptr);
+                      int uniform_only = 0, int *clear = nullptr);
 // The same for kTcSplitF16x3 tables (tc_half.cu; bn = 128).
 cudaError_t launch_tc_half(const ProbTable &tab, int total_units,
                            const int *unit_map, const int *flags, void *pack_base,
@@ -306,7 +303,7 @@ cudaError_t launch_tc_half(const ProbTable &tab, int total_units,
 // (64 or 128) bytes x box_rows rows with the matching swizzle, into `map` (128
 // bytes, 64-byte aligned).
 cudaError_t encode_pack_map(void *map, void *base, int64_t rows, int bkb, int box_rows = 128);
-// Tensor map over C for the tensor-core epilogue's tiled stores (128 bytes
+// Tensor map over an FP32 matrix in boxes of 32 x 32 (128 bytes
 // written to `map`); usable where tc_c_map_ok holds.
 bool tc_c_map_ok(const float *C, int64_t n, int64_t p);
 cudaError_t encode_c_map(void *map, float *C, int64_t n, int64_t p);

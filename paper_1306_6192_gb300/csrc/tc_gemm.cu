@@ -16,7 +16,7 @@
 // and everything below are this library's GB300 design, not the paper's (its
 // kernels, Listings 2-4, use CUDA cores only).
 //
-// Kernel structure (persistent, one CTA per SM, 192 threads):
+// Kernel structure (persistent, one CTA per SM, 320 threads):
 //   warp 0    TMEM allocation; lane 0 issues TMA loads of the A and B pack
 //             tiles (all parts) of each K step into a STAGES-deep shared-
 //             memory ring (mbarrier "full" with transaction bytes).
@@ -24,12 +24,15 @@
 //             instruction) - three per K step for the split kind, one for
 //             e4m3 - and commits each stage back to the producer ("empty")
 //             and each finished tile to the epilogue ("acc_full").
-//   warps 2-5 epilogue: tcgen05.ld of the accumulator (each warp reads its
-//             32 TMEM lanes = 32 rows), exact power-of-two unscaling, each
-//             32 x 32 block through shared memory: one tiled TMA store per
-//             block where the host gave C a tensor map (the store clips the
-//             edges), else whole 128-byte-line stores of each row (edge rows
-//             and columns predicated); then "acc_empty".
+//   warps 2-9 epilogue: tcgen05.ld of the accumulator (each warp reads its
+//             32 TMEM lanes = 32 rows, in half of the columns), exact
+//             power-of-two unscaling, then whole 32-byte sectors from a
+//             lane's registers to its row, or, where C's rows are off that
+//             alignment, through shared memory to 64-byte pieces of a row
+//             (edge rows and columns predicated); then "acc_empty".  Four
+//             warps with a block of 32 columns staged for a TMA store took
+//             16 us a 128 x 256 tile, longer than its MMAs below K = 5000
+//             (e4m3 4096 x 1024 x 4096 70 us, 4096^3 85; now 45 and 64).
 // Two accumulators of 256 TMEM columns each (four of 128 in the 128-wide
 // layouts) let the epilogue of one tile overlap the mainloop of the next.
 // The work units (tiles, or K parts of split tiles) of all problems of a
@@ -62,7 +65,8 @@
 namespace mm {
 namespace {
 
-constexpr int kThreads = 192;
+constexpr int kThreads = 320;
+constexpr int kEpiThreads = 256;
 constexpr uint32_t kTmemCols = 512;         // all of TMEM: the accumulators
 constexpr int kBoxRows = 128;               // TMA box height (rows of the pack)
 constexpr uint64_t kWaitLimitNs = 4000000000ull;
@@ -70,14 +74,14 @@ constexpr uint64_t kDrainLimitNs = 200000000ull;
 
 using namespace tcx;
 
-// AND of `v` over the 128 epilogue threads (named barrier 1): every thread
-// arrives, so the four warps leave the tile loop together.
+// AND of `v` over the epilogue threads (named barrier 1): every thread
+// arrives, so the warps leave the tile loop together.
 __device__ __forceinline__ bool epilogue_all(bool v) {
   uint32_t r;
   asm volatile(
       "{\n\t.reg .pred p, q;\n\t"
       "setp.ne.u32 q, %1, 0;\n\t"
-      "bar.red.and.pred p, 1, 128, q;\n\t"
+      "bar.red.and.pred p, 1, 256, q;\n\t"
       "selp.u32 %0, 1, 0, p;\n\t}\n"
       : "=r"(r)
       : "r"((uint32_t)v)
@@ -108,7 +112,7 @@ __device__ __forceinline__ bool skip_unit(const SplitProb &pr, int uniform_only,
 }
 
 __device__ __forceinline__ void epilogue_sync() {
-  asm volatile("bar.sync 1, 128;" ::: "memory");
+  asm volatile("bar.sync 1, 256;" ::: "memory");
 }
 
 // Shared-memory layout of one instantiation: STAGES ring stages of BKB bytes
@@ -129,28 +133,25 @@ struct TcLayout {
   // that the epilogues of short tiles can lag the MMAs by several tiles
   static constexpr int kNumAcc = (int)kTmemCols / kMaxBN;
   static constexpr int kNumBars = 2 * STAGES + 2 * kNumAcc + 1;  // full, empty, acc f/e, drain
-  static constexpr int kColExpOffset = kBarOffset + kNumBars * 8 + 16;  // int[kNumAcc][kMaxBN]
+  static constexpr int kColExpOffset = (kBarOffset + kNumBars * 8 + 31) & ~15;  // int[kNumAcc][kMaxBN]
   static constexpr int kLastOffset = kColExpOffset + kNumAcc * kMaxBN * 4;  // last-part flag
-  // epilogue staging: one 32 x 33 float block per epilogue warp
-  // epilogue staging, one 5 KB region per epilogue warp (1024-byte aligned):
-  // a dense 32 x 32 FP32 block with a 128-byte swizzle for the tiled stores,
-  // or rows of 33 floats for the plain stores
-  static constexpr int kStageStride = 5120;
-  static constexpr int kStageOffset = (kLastOffset + 16 + 1023) & ~1023;
-  static constexpr int kSmemBytes = kStageOffset + 4 * kStageStride + 1024;  // + align slack
+  // staging of the plain stores: 32 rows of 17 floats per epilogue warp
+  static constexpr int kStageFloats = 32 * 17;
+  static constexpr int kStageOffset = kLastOffset + 16;
+  static constexpr int kSmemBytes = kStageOffset + 8 * kStageFloats * 4 + 1024;  // + align slack
 };
 
-// ONE: the table is one product carried in the launch (tab.one, one_cmap);
-// else dev_probs and many_cmaps.  An instantiation each: with one pointer for
+// ONE: the table is one product carried in the launch (tab.one);
+// else dev_probs.  An instantiation each: with one pointer for
 // both, the roles read a device table through generic loads again and again
 // (the FP64 emulation of 4096^3 4133 us instead of 4079).
 template <int BKB, int STAGES, int KIND, int MAXBN, bool ONE>
 __global__ void __launch_bounds__(kThreads, 1)
-tc_gemm_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_constant__ CUtensorMap one_cmap,
+tc_gemm_kernel(const __grid_constant__ CUtensorMap tmap,
                const __grid_constant__ ProbTable tab, const SplitProb *__restrict__ dev_probs,
                const int *__restrict__ unit_map,
                const int *__restrict__ flags, int total_units, const int *__restrict__ order,
-               int uniform_only, const CUtensorMap *__restrict__ many_cmaps, int *clear, int *err) {
+               int uniform_only, int *clear, int *err) {
   using L = TcLayout<BKB, STAGES, KIND, MAXBN>;
   extern __shared__ uint8_t smem_raw[];
   const uint32_t raw = smem_u32(smem_raw);
@@ -172,7 +173,6 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_constant__
   if (ONE) table_products(tab, &shared_one);
   const SplitProb *__restrict__ probs = ONE ? &shared_one : dev_probs;
   const int nprobs = ONE ? 1 : tab.n;
-  const CUtensorMap *c_maps = ONE ? &one_cmap : many_cmaps;
 
   if (warp == 0) {
     tmem_alloc(smem_u32(tmem_holder), kTmemCols);
@@ -185,7 +185,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_constant__
     }
     for (int a = 0; a < L::kNumAcc; a++) {
       mbar_init(accf_bar(a), 1);
-      mbar_init(acce_bar(a), 4 * 32);
+      mbar_init(acce_bar(a), kEpiThreads);
     }
     mbar_init(drain_bar, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -354,7 +354,8 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_constant__
     const int row = q * 32 + lane;
     int acc = 0;
     uint32_t acc_phase = 0;
-    const int et = threadIdx.x - 64;  // 0..127 over the epilogue warps
+    const int et = threadIdx.x - 64;  // over the epilogue warps
+    const int half = (warp - 2) >> 2;  // which half of the columns
     for (int ui = i_first; ui < i_end; ui += i_step) {
       const int u = ulist ? ulist[ui] : ui;
       const UnitCoord tc = decode_unit(probs, nprobs, unit_map, u);
@@ -364,21 +365,29 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_constant__
       // operands packed without scaling (flags) take exponent 0
       const int fl = flags ? flags[tc.g] : (kFlagScaleA | kFlagScaleB);
       int *cexp = colexp + acc * MAXBN;
-      for (int c = et; c < pr.bn; c += 128) {
+      bool small = true;  // every exponent within +-60
+      for (int c = et; c < pr.bn; c += kEpiThreads) {
         const int64_t j = (int64_t)tc.nt * pr.bn + c;
         cexp[c] = (j < pr.p && (fl & kFlagScaleB)) ? kind_exponent<KIND>(pr.tB[j]) : 0;
+        small &= abs(cexp[c]) <= 60;
       }
-      const bool ok = mbar_wait(accf_bar(acc), acc_phase, err, 4, true, kWaitLimitNs);
-      if (!epilogue_all(ok)) break;  // also orders the cexp writes before the reads
-      tc_fence_after();
       const int64_t i = (int64_t)tc.mt * kTcBM + row;
       const bool row_ok = i < pr.n;
       const int si = (row_ok && (fl & kFlagScaleA)) ? kind_exponent<KIND>(pr.sA[i]) : 0;
-      float *buf = stage_buf + q * (L::kStageStride / 4);  // this warp's 32 x 32 block
-      const CUtensorMap *cmap = (c_maps != nullptr && pr.c_tma > 0) ? c_maps + (pr.c_tma - 1)
-                                                                     : nullptr;
+      // (also orders the cexp writes before the reads)
+      small = epilogue_all(small && abs(si) <= 60);
+      const float rfac = __int_as_float((si + 127) << 23);  // where small
+      const bool ok = mbar_wait(accf_bar(acc), acc_phase, err, 4, true, kWaitLimitNs);
+      if (!epilogue_all(ok)) break;
+      tc_fence_after();
+      float *buf = stage_buf + (warp - 2) * L::kStageFloats;
       const int64_t row0 = (int64_t)tc.mt * kTcBM + q * 32;  // first row of the warp
       const uint32_t tacc = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(acc * MAXBN);
+      const int c_first = half * (pr.bn / 2), c_end = c_first + pr.bn / 2;
+      // vectors of 8 or 4 columns, wholly inside or outside C and D
+      const uintptr_t at = reinterpret_cast<uintptr_t>(pr.C) |
+                           (pr.epi.on == 2 ? reinterpret_cast<uintptr_t>(pr.epi.D) & 15u : 0u);
+      const int vec = (at & 15u) != 0 || (pr.p & 3) != 0 ? 0 : ((at & 31u) == 0 && (pr.p & 7) == 0 ? 8 : 4);
       // part of a split tile: a partial slot holds bn/4 groups of 4 columns,
       // each group 128 rows x 4 floats, so that a warp's 16-byte accesses to
       // one group (32 rows) are 512 consecutive bytes
@@ -392,7 +401,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_constant__
       if (tc.h >= 0) {
         float4 *mine = reinterpret_cast<float4 *>(
                            pr.part + ((size_t)st * split_s + tc.h) * slot_floats) + row;
-        for (int c = 0; c < pr.bn; c += 32) {
+        for (int c = c_first; c < c_end; c += 32) {
           uint32_t v[32];
           __syncwarp();
           tmem_ld_32x32b_x32(tacc + (uint32_t)c, v);
@@ -413,139 +422,139 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_constant__
           if (et == 0) pr.cnt[st] = 0;  // ready for the next launch
         }
       }
-      for (int c = 0; c < pr.bn && store; c += 32) {
+      for (int c = c_first; c < c_end && store; c += 32) {
         uint32_t v[32];
         __syncwarp();  // tcgen05.ld is warp-collective: reconverge first
         tmem_ld_32x32b_x32(tacc + (uint32_t)c, v);
         tmem_ld_wait();
         if (tc.h >= 0) {
           // sum of the parts in order 0..split_s-1 (this part's from TMEM);
-          // the loads of all other parts of the chunk are issued first
-          float4 x[kMaxSplit][8];
+          // the loads of all other parts of half a chunk are issued first
 #pragma unroll
-          for (int hh = 0; hh < kMaxSplit; hh++) {
-            if (hh < split_s && hh != tc.h) {
-              const float4 *src = slots + (size_t)hh * (slot_floats / 4) + (size_t)(c >> 2) * kTcBM;
-#pragma unroll
-              for (int e = 0; e < 8; e++) x[hh][e] = __ldcg(src + (size_t)e * kTcBM);
-            }
-          }
-#pragma unroll
-          for (int e = 0; e < 8; e++) {
-            float4 sum = make_float4(0.f, 0.f, 0.f, 0.f);
+          for (int e0 = 0; e0 < 8; e0 += 4) {
+            float4 x[kMaxSplit][4];
 #pragma unroll
             for (int hh = 0; hh < kMaxSplit; hh++) {
-              if (hh >= split_s) break;
-              const float4 y = hh == tc.h ? make_float4(__uint_as_float(v[4 * e]),
-                                                        __uint_as_float(v[4 * e + 1]),
-                                                        __uint_as_float(v[4 * e + 2]),
-                                                        __uint_as_float(v[4 * e + 3]))
-                                          : x[hh][e];
-              if (hh == 0) {
-                sum = y;
-              } else {
-                sum.x += y.x;
-                sum.y += y.y;
-                sum.z += y.z;
-                sum.w += y.w;
+              if (hh < split_s && hh != tc.h) {
+                const float4 *src = slots + (size_t)hh * (slot_floats / 4) + (size_t)((c >> 2) + e0) * kTcBM;
+#pragma unroll
+                for (int e = 0; e < 4; e++) x[hh][e] = __ldcg(src + (size_t)e * kTcBM);
               }
             }
-            v[4 * e] = __float_as_uint(sum.x);
-            v[4 * e + 1] = __float_as_uint(sum.y);
-            v[4 * e + 2] = __float_as_uint(sum.z);
-            v[4 * e + 3] = __float_as_uint(sum.w);
+#pragma unroll
+            for (int e = 0; e < 4; e++) {
+              uint32_t *w = v + 4 * (e0 + e);
+              float4 sum = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+              for (int hh = 0; hh < kMaxSplit; hh++) {
+                if (hh >= split_s) break;
+                const float4 y = hh == tc.h ? make_float4(__uint_as_float(w[0]), __uint_as_float(w[1]),
+                                                          __uint_as_float(w[2]), __uint_as_float(w[3]))
+                                            : x[hh][e];
+                if (hh == 0) {
+                  sum = y;
+                } else {
+                  sum.x += y.x;
+                  sum.y += y.y;
+                  sum.z += y.z;
+                  sum.w += y.w;
+                }
+              }
+              w[0] = __float_as_uint(sum.x);
+              w[1] = __float_as_uint(sum.y);
+              w[2] = __float_as_uint(sum.z);
+              w[3] = __float_as_uint(sum.w);
+            }
           }
         }
         const int64_t j0 = (int64_t)tc.nt * pr.bn + c;
         if (j0 >= pr.p) continue;  // the same for the whole warp
         const int *ce = cexp + c;
-        if (cmap) {
-          // the block into the dense staging area, 16-byte chunk k of row
-          // `lane` at chunk k ^ (lane & 7) (the 128-byte swizzle of the map;
-          // the writes of one instruction then spread over all banks), and
-          // one tiled store of it; the area is rewritten only after the
-          // previous store has read it
-          if (lane == 0) bulk_wait_read_all();
-          __syncwarp();
-          float4 *rowp = reinterpret_cast<float4 *>(buf + lane * 32);
+        // exact: a power of two, of two factors where both are small
+        if (small) {
 #pragma unroll
-          for (int k = 0; k < 8; k++)
-            rowp[k ^ (lane & 7)] =
-                make_float4(scale_pow2(__uint_as_float(v[4 * k]), si + ce[4 * k]),
-                            scale_pow2(__uint_as_float(v[4 * k + 1]), si + ce[4 * k + 1]),
-                            scale_pow2(__uint_as_float(v[4 * k + 2]), si + ce[4 * k + 2]),
-                            scale_pow2(__uint_as_float(v[4 * k + 3]), si + ce[4 * k + 3]));
+          for (int k = 0; k < 32; k += 4) {
+            const int4 e4 = *reinterpret_cast<const int4 *>(ce + k);
+            v[k] = __float_as_uint(__uint_as_float(v[k]) * (rfac * __int_as_float((e4.x + 127) << 23)));
+            v[k + 1] = __float_as_uint(__uint_as_float(v[k + 1]) * (rfac * __int_as_float((e4.y + 127) << 23)));
+            v[k + 2] = __float_as_uint(__uint_as_float(v[k + 2]) * (rfac * __int_as_float((e4.z + 127) << 23)));
+            v[k + 3] = __float_as_uint(__uint_as_float(v[k + 3]) * (rfac * __int_as_float((e4.w + 127) << 23)));
+          }
+        } else {
+#pragma unroll
+          for (int k = 0; k < 32; k++) v[k] = __float_as_uint(scale_pow2(__uint_as_float(v[k]), si + ce[k]));
+        }
+        if (vec != 0) {
+          // this thread's row: its 32 values of D in eight 16-byte loads in
+          // flight, the results in whole sectors
+          if (!row_ok) continue;
           if (pr.epi.on != 0) {
-            // C = alpha (A.B) + beta D on this thread's row of the block, in
-            // place in the staging area: the row's 32 values of D in eight
-            // 16-byte loads in flight (p % 4 == 0 and a 16-byte aligned D,
-            // so a vector is wholly inside or outside C's columns)
-            const int64_t i = row0 + lane;
             const float al = pr.epi.alpha, be = pr.epi.beta;
             if (pr.epi.on == 2) {
               const float4 *drow = reinterpret_cast<const float4 *>(pr.epi.D + i * pr.p + j0);
               float4 dq[8];
 #pragma unroll
               for (int k = 0; k < 8; k++)
-                dq[k] = (i < pr.n && j0 + 4 * k < pr.p) ? drow[k] : make_float4(0.f, 0.f, 0.f, 0.f);
+                dq[k] = j0 + 4 * k < pr.p ? drow[k] : make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
               for (int k = 0; k < 8; k++) {
-                const float4 x = rowp[k ^ (lane & 7)];
-                rowp[k ^ (lane & 7)] = make_float4(fmaf(al, x.x, be * dq[k].x), fmaf(al, x.y, be * dq[k].y),
-                                                   fmaf(al, x.z, be * dq[k].z), fmaf(al, x.w, be * dq[k].w));
+                v[4 * k] = __float_as_uint(fmaf(al, __uint_as_float(v[4 * k]), be * dq[k].x));
+                v[4 * k + 1] = __float_as_uint(fmaf(al, __uint_as_float(v[4 * k + 1]), be * dq[k].y));
+                v[4 * k + 2] = __float_as_uint(fmaf(al, __uint_as_float(v[4 * k + 2]), be * dq[k].z));
+                v[4 * k + 3] = __float_as_uint(fmaf(al, __uint_as_float(v[4 * k + 3]), be * dq[k].w));
               }
             } else {
 #pragma unroll
-              for (int k = 0; k < 8; k++) {
-                const float4 x = rowp[k];
-                rowp[k] = make_float4(al * x.x, al * x.y, al * x.z, al * x.w);
-              }
+              for (int k = 0; k < 32; k++) v[k] = __float_as_uint(al * __uint_as_float(v[k]));
             }
           }
-          fence_proxy_async_shared();
-          __syncwarp();
-          if (lane == 0 && row0 < pr.n) {  // a block wholly below C is not stored
-            tma_store_2d(cmap, smem_u32(buf), (int)j0, (int)row0);
-            bulk_commit();
+          float *dst = pr.C + i * pr.p + j0;
+          if (vec == 8) {
+#pragma unroll
+            for (int k = 0; k < 32; k += 8)
+              if (j0 + k < pr.p) store8(dst + k, reinterpret_cast<const float *>(v + k));
+          } else {
+#pragma unroll
+            for (int k = 0; k < 32; k += 4)
+              if (j0 + k < pr.p)
+                *reinterpret_cast<float4 *>(dst + k) =
+                    make_float4(__uint_as_float(v[k]), __uint_as_float(v[k + 1]), __uint_as_float(v[k + 2]),
+                                __uint_as_float(v[k + 3]));
           }
           continue;
         }
-        // unscale this thread's row of the 32 x 32 block into shared memory,
-        // then write the block row by row: each store is 32 consecutive
-        // columns of one row, a whole 128-byte line
+        // through shared memory, 16 columns at a time: two rows a store
+        const int64_t left = pr.n - row0;
+        const int rows = left < 32 ? (int)left : 32;
 #pragma unroll
-        for (int e = 0; e < 32; e++)
-          buf[lane * 33 + e] = scale_pow2(__uint_as_float(v[e]), si + ce[e]);
-        __syncwarp();
-        const int64_t j = j0 + lane;
-        if (j < pr.p) {
-          float *dst = pr.C + row0 * pr.p + j;
-          const int64_t left = pr.n - row0;
-          const int rows = left < 32 ? (int)left : 32;
+        for (int hc = 0; hc < 32; hc += 16) {
+          __syncwarp();
+#pragma unroll
+          for (int e = 0; e < 16; e++) buf[lane * 17 + e] = __uint_as_float(v[hc + e]);
+          __syncwarp();
+          const int64_t j = j0 + hc + (lane & 15);
+          if (j >= pr.p) continue;
+          const int64_t x0 = (row0 + (lane >> 4)) * pr.p + j;
+          const float *src = buf + (lane >> 4) * 17 + (lane & 15);
           if (pr.epi.on == 0) {
-#pragma unroll 8
-            for (int r = 0; r < rows; r++, dst += pr.p) __stcs(dst, buf[r * 33 + lane]);
+#pragma unroll
+            for (int r = 0; r < 32; r += 2)
+              if (r + (lane >> 4) < rows) __stcs(pr.C + x0 + r * (int64_t)pr.p, src[r * 17]);
           } else {
-            // C = alpha (A.B) + beta D, sixteen rows at a time: their values
-            // of D are loaded before any of them is stored (D may be C)
-            const float *dcol = pr.epi.D + row0 * pr.p + j;
+            // C = alpha (A.B) + beta D: a thread's values of D are loaded
+            // before any of its entries is stored (D may be C)
+            float dv[16];
 #pragma unroll
-            for (int h = 0; h < 32; h += 16) {
-              float dv[16];
+            for (int r = 0; r < 32; r += 2)
+              dv[r / 2] = (pr.epi.on == 2 && r + (lane >> 4) < rows) ? pr.epi.D[x0 + r * (int64_t)pr.p] : 0.f;
 #pragma unroll
-              for (int r = 0; r < 16; r++)
-                dv[r] = (pr.epi.on == 2 && h + r < rows) ? dcol[(int64_t)(h + r) * pr.p] : 0.f;
-#pragma unroll
-              for (int r = 0; r < 16; r++)
-                if (h + r < rows)
-                  __stcs(dst + (int64_t)(h + r) * pr.p,
-                         pr.epi.on == 2
-                             ? fmaf(pr.epi.alpha, buf[(h + r) * 33 + lane], pr.epi.beta * dv[r])
-                             : pr.epi.alpha * buf[(h + r) * 33 + lane]);
-            }
+            for (int r = 0; r < 32; r += 2)
+              if (r + (lane >> 4) < rows)
+                __stcs(pr.C + x0 + r * (int64_t)pr.p,
+                       pr.epi.on == 2 ? fmaf(pr.epi.alpha, src[r * 17], pr.epi.beta * dv[r / 2])
+                                      : pr.epi.alpha * src[r * 17]);
           }
         }
-        __syncwarp();
       }
       tc_fence_before();
       mbar_arrive(acce_bar(acc));
@@ -554,9 +563,6 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_constant__
         acc_phase ^= 1u;
       }
     }
-    // the tiled stores have read shared memory and completed
-    if (lane == 0) bulk_wait_all();
-    __syncwarp();
   }
 
   tc_fence_before();
@@ -600,9 +606,9 @@ cudaError_t encode_pack_map(void *map, void *base, int64_t rows, int bkb, int bo
   return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
 }
 
-// 2-D map over C (n rows of p FP32, row-major) for the epilogue's tiled
-// stores: boxes of 32 x 32 with a 128-byte swizzle.  Needs a 16-byte aligned
-// C and p a multiple of 4.
+// 2-D map over an FP32 matrix (n rows of p, row-major), boxes of 32 x 32 with a
+// 128-byte swizzle (the D of tc_half.cu's epilogue).  Needs 16-byte alignment
+// and p a multiple of 4.
 bool tc_c_map_ok(const float *C, int64_t n, int64_t p) {
   return (reinterpret_cast<uintptr_t>(C) & 15u) == 0 && (p & 3) == 0 && n > 0 && p > 0 &&
          n <= 0x7fffffffLL && p <= 0x7fffffffLL;
@@ -629,11 +635,11 @@ namespace {
 template <int BKB, int STAGES, int KIND, int MAXBN, bool ONE = false>
 cudaError_t launch_tc_t(const ProbTable &tab, const int *unit_map, const int *flags, int total_units, void *pack_base, int64_t pack_rows,
                         int grid, int *d_err, cudaStream_t s, const int *order,
-                        int uniform_only, const void *c_maps, int *clear) {
+                        int uniform_only, int *clear) {
   if constexpr (KIND != kTcE4m3 && !ONE)
     if (tab.dev == nullptr)
       return launch_tc_t<BKB, STAGES, KIND, MAXBN, true>(tab, unit_map, flags, total_units, pack_base, pack_rows,
-                                                         grid, d_err, s, order, uniform_only, c_maps, clear);
+                                                         grid, d_err, s, order, uniform_only, clear);
   using L = TcLayout<BKB, STAGES, KIND, MAXBN>;
   static_assert(L::kSmemBytes + sizeof(SplitProb) <= 232448, "shared memory budget");
   // one CTA per SM: the kernel allocates all 512 TMEM columns
@@ -649,17 +655,11 @@ cudaError_t launch_tc_t(const ProbTable &tab, const int *unit_map, const int *fl
   cudaError_t e = encode_pack_map(&map, pack_base, pack_rows, BKB);
   if (e != cudaSuccess) return e;
   TraceScope ts(KIND == kTcE4m3 ? "fp8_tc" : "split_tc", s);
-  // a product carried in the launch brings its C's map along, too
-  CUtensorMap one_cmap = {};
-  if (tab.dev == nullptr && tab.one.c_tma > 0) {
-    e = encode_c_map(&one_cmap, tab.one.C, tab.one.n, tab.one.p);
-    if (e != cudaSuccess) return e;
-  }
   // (as a dependent of the digit kernel the FP64 emulation's launch made its call
   // 2.5% slower, 4090 us against 3990 at 4096^3)
   return launch_pdl_if(ONE, tc_gemm_kernel<BKB, STAGES, KIND, MAXBN, ONE>, (unsigned)grid, kThreads,
-                       L::kSmemBytes, s, map, one_cmap, tab, tab.dev, unit_map, flags, total_units, order, uniform_only,
-                    static_cast<const CUtensorMap *>(c_maps), clear, d_err);
+                       L::kSmemBytes, s, map, tab, tab.dev, unit_map, flags, total_units, order, uniform_only, clear,
+                       d_err);
 }
 
 }  // namespace
@@ -769,13 +769,13 @@ size_t tc_tail_bytes(const TcTail &t, int64_t tiles, int bn) {
 cudaError_t launch_tc(TcKind kind, const ProbTable &tab, int total_units, const int *unit_map,
                       const int *flags, void *pack_base, int64_t pack_rows,
                       const TcConfig &cfg, int *d_err, cudaStream_t s, const int *order,
-                      int uniform_only, const void *c_maps, int *clear) {
+                      int uniform_only, int *clear) {
   if (total_units <= 0) return cudaSuccess;
   if (pack_rows <= 0 || pack_rows > 0x7fffffffLL) return cudaErrorInvalidValue;
   const int grid = tc_launch_grid(cfg, total_units);
   const int *mp = unit_map;
 #define MM_TC_ARGS \
-  tab, mp, flags, total_units, pack_base, pack_rows, grid, d_err, s, order, uniform_only, c_maps, clear
+  tab, mp, flags, total_units, pack_base, pack_rows, grid, d_err, s, order, uniform_only, clear
   cudaError_t e = cudaErrorInvalidValue;
   const bool narrow = cfg.max_bn <= 128;  // every N tile of the table fits 128
   if (kind == kTcE4m3) e = launch_tc_t<128, 4, kTcE4m3, 256>(MM_TC_ARGS);

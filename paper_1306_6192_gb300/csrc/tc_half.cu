@@ -132,13 +132,6 @@ __device__ __forceinline__ bool epi_wait(uint32_t bar, uint32_t parity, int *err
   }
 }
 
-// Eight consecutive floats at a 32-byte boundary: one whole sector a lane.
-__device__ __forceinline__ void store8(float *dst, const float *v) {
-  asm volatile("st.global.v8.f32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(dst), "f"(v[0]), "f"(v[1]),
-               "f"(v[2]), "f"(v[3]), "f"(v[4]), "f"(v[5]), "f"(v[6]), "f"(v[7])
-               : "memory");
-}
-
 // Instruction descriptor: FP32 accumulators, K-major fp16 (fmt 0) or bf16
 // (fmt 1) operands, M = 128.
 __device__ __forceinline__ uint32_t idesc_f16(uint32_t fmt, int bn) {

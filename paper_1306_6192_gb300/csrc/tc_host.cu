@@ -145,12 +145,8 @@ mm_status run_tc_groups(Scratch &ws, const mm_problem *probs, int count, cudaStr
     order_ints += orders[gi].size();
   }
   const size_t tab_bytes = (ntab * sizeof(SplitProb) + 15) & ~(size_t)15;
-  // tensor maps over the C matrices for the epilogue's tiled stores, for
-  // tables of up to kMaxCMaps products (each map is encoded on the host)
-  constexpr size_t kMaxCMaps = 8192, kMapBytes = 128;
-  const size_t cmap_rel = (tab_bytes + order_ints * sizeof(int) + 63) & ~(size_t)63;
-  const size_t cmap_bytes = ntab <= kMaxCMaps ? ntab * kMapBytes : 0;
-  const size_t map_off = (tab_off + cmap_rel + cmap_bytes + 255) & ~(size_t)255;
+  const size_t blob_bytes = tab_bytes + order_ints * sizeof(int);
+  const size_t map_off = (tab_off + blob_bytes + 255) & ~(size_t)255;
   const size_t tpart_off = (map_off + map_ints * sizeof(int) + 255) & ~(size_t)255;
   const size_t need = tpart_off + tail_parts;
   cudaError_t e = ws.reserve(need, s);
@@ -185,26 +181,9 @@ mm_status run_tc_groups(Scratch &ws, const mm_problem *probs, int count, cudaStr
   }
   SplitProb *d_tab = reinterpret_cast<SplitProb *>(base + tab_off);
   int *d_orders = reinterpret_cast<int *>(base + tab_off + tab_bytes);
-  const void *d_cmaps = cmap_bytes ? static_cast<const void *>(base + tab_off + cmap_rel) : nullptr;
-  // C matrices that the tensor-core kernel may write with tiled stores
-  auto tiled_c = [](const SplitProb &sp) {
-    // the epilogue C = alpha (A.B) + beta D loads D in 16-byte vectors beside
-    // the tiled stores (a D off that alignment: plain stores); tc_half.cu
-    // stores whole sectors from registers
-    return sp.hx == nullptr && (sp.epi.on != 2 || (reinterpret_cast<uintptr_t>(sp.epi.D) & 15u) == 0) &&
-           tc_c_map_ok(sp.C, sp.n, sp.p);
-  };
-  if (single) {
-    all[0].c_tma = tiled_c(all[0]) ? 1 : 0;
-  } else {
-    // one copy: the table, the CTAs' unit lists, the C tensor maps
-    std::vector<uint8_t> blob(cmap_rel + cmap_bytes, 0);
-    for (size_t k = 0; cmap_bytes && k < ntab; k++) {
-      SplitProb &sp = all[k];
-      if (tiled_c(sp) &&
-          encode_c_map(blob.data() + cmap_rel + k * kMapBytes, sp.C, sp.n, sp.p) == cudaSuccess)
-        sp.c_tma = (int32_t)k + 1;
-    }
+  if (!single) {
+    // one copy: the table, the CTAs' unit lists
+    std::vector<uint8_t> blob(blob_bytes, 0);
     std::memcpy(blob.data(), all.data(), all.size() * sizeof(SplitProb));
     size_t at = tab_bytes;
     for (auto &o : orders) {
@@ -254,7 +233,7 @@ mm_status run_tc_groups(Scratch &ws, const mm_problem *probs, int count, cudaStr
               ? launch_tc_half(dt, (int)G.units, tile_map, flags, base, rows,
                                tc_launch_grid(G.cfg, G.units), g_ctx.d_err, s, order, clear)
               : launch_tc(G.kind, dt, (int)G.units, tile_map, flags, base, rows, G.cfg, g_ctx.d_err,
-                          s, order, 0, d_cmaps, clear);
+                          s, order, 0, clear);
     if (e != cudaSuccess) {
       ws.words_epoch = 0;  // the words may be left set
       return note_cuda(e);

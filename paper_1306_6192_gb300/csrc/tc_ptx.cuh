@@ -192,35 +192,15 @@ __device__ __forceinline__ uint32_t make_idesc(int bn) {
          ((uint32_t)(kTcBM >> 4) << 24);
 }
 
-// Tiled bulk store of a box from this CTA's shared memory to global memory
-// through a tensor map (elements outside the tensor are not written), in this
-// thread's current bulk group.  x (the inner coordinate) times the element
-// size must be a multiple of 16 bytes and neither coordinate negative; the
-// shared-memory writes it reads must precede fence_proxy_async_shared() by
-// the writing threads and a barrier with the issuing thread.
-__device__ __forceinline__ void tma_store_2d(const CUtensorMap *map, uint32_t src, int x, int y) {
-  asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.tile.bulk_group [%0, {%2, %3}], [%1];" ::"l"(
-                   reinterpret_cast<uint64_t>(map)),
-               "r"(src), "r"(x), "r"(y)
+// Eight consecutive floats at a 32-byte boundary: one whole sector a lane.
+__device__ __forceinline__ void store8(float *dst, const float *v) {
+  asm volatile("st.global.v8.f32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(dst), "f"(v[0]), "f"(v[1]),
+               "f"(v[2]), "f"(v[3]), "f"(v[4]), "f"(v[5]), "f"(v[6]), "f"(v[7])
                : "memory");
 }
 
 __device__ __forceinline__ void fence_proxy_async_shared() {
   asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-}
-
-__device__ __forceinline__ void bulk_commit() {
-  asm volatile("cp.async.bulk.commit_group;" ::: "memory");
-}
-
-// This thread's bulk groups have finished reading shared memory.
-__device__ __forceinline__ void bulk_wait_read_all() {
-  asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
-}
-
-// This thread's bulk groups have completed.
-__device__ __forceinline__ void bulk_wait_all() {
-  asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
 }
 
 // Paired FP32 arithmetic (two independent lanes in one 64-bit register, the
