@@ -125,9 +125,11 @@ __device__ __forceinline__ float pow2f(int e) { return scale_pow2(1.0f, e); }
 // which order like the magnitudes) into the problem's sA / tB (zeroed before
 // the launch).  Items of a problem, from the prefix `split_from` of its entry
 // in the blockwise table: ceil(n / 8) items of 8 rows of A (a warp per row,
-// 16-byte loads where the row allows), then strips of 128 columns x 256 rows
-// of B (four columns per lane), merged with atomicMax.
-constexpr int kMaxRows = 8, kMaxStrip = 128, kMaxChunk = 256;
+// 16-byte loads where the row allows), then strips of 128 columns x 64 rows
+// of B (four columns per lane), merged with atomicMax.  Bound by reading A and
+// B: eight loads in flight a lane (one at a time: 4096 x 1024 x 4096, 34 MB, 25 us,
+// now 13; 4096^3, 134 MB, 39).
+constexpr int kMaxRows = 8, kMaxStrip = 128, kMaxChunk = 64;
 
 __host__ __device__ inline int64_t max_items(int64_t n, int64_t m, int64_t p) {
   return (n + kMaxRows - 1) / kMaxRows +
@@ -155,8 +157,10 @@ fp8blk_max_kernel(const SplitProb *__restrict__ probs, int nprobs) {
     uint32_t mx = 0;
     if ((reinterpret_cast<uintptr_t>(pr.A) & 15u) == 0 && (pr.m & 3) == 0) {
       const float4 *r4 = reinterpret_cast<const float4 *>(row);
+#pragma unroll 8
       for (int64_t k = lane; k < pr.m / 4; k += 32) mx = max(mx, absmax4(__ldg(r4 + k)));
     } else {
+#pragma unroll 8
       for (int64_t k = lane; k < pr.m; k += 32) mx = max(mx, __float_as_uint(row[k]) & 0x7fffffffu);
     }
 #pragma unroll
@@ -170,20 +174,28 @@ fp8blk_max_kernel(const SplitProb *__restrict__ probs, int nprobs) {
   const int64_t c0 = (b % strips) * kMaxStrip + 4 * lane, r0 = (b / strips) * kMaxChunk;
   const bool vec = (reinterpret_cast<uintptr_t>(pr.B) & 15u) == 0 && (pr.p & 3) == 0;
   uint32_t mx[4] = {0, 0, 0, 0};
-  for (int r = warp; r < kMaxChunk; r += 8) {
-    const int64_t k = r0 + r;
-    if (k >= pr.m) break;
-    const float *src = pr.B + k * pr.p + c0;
-    if (vec && c0 + 4 <= pr.p) {
-      const float4 v = __ldg(reinterpret_cast<const float4 *>(src));
-      mx[0] = max(mx[0], __float_as_uint(v.x) & 0x7fffffffu);
-      mx[1] = max(mx[1], __float_as_uint(v.y) & 0x7fffffffu);
-      mx[2] = max(mx[2], __float_as_uint(v.z) & 0x7fffffffu);
-      mx[3] = max(mx[3], __float_as_uint(v.w) & 0x7fffffffu);
-    } else {
+  if (vec) {
+    float4 v[kMaxChunk / 8];
+#pragma unroll
+    for (int r = 0; r < kMaxChunk / 8; r++) {
+      const int64_t k = r0 + warp + 8 * r;
+      v[r] = k < pr.m && c0 < pr.p ? __ldg(reinterpret_cast<const float4 *>(pr.B + k * pr.p + c0))
+                                   : make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+#pragma unroll
+    for (int r = 0; r < kMaxChunk / 8; r++) {
+      mx[0] = max(mx[0], absb(v[r].x));
+      mx[1] = max(mx[1], absb(v[r].y));
+      mx[2] = max(mx[2], absb(v[r].z));
+      mx[3] = max(mx[3], absb(v[r].w));
+    }
+  } else {
+#pragma unroll 2
+    for (int r = 0; r < kMaxChunk / 8; r++) {
+      const int64_t k = r0 + warp + 8 * r;
 #pragma unroll
       for (int e = 0; e < 4; e++)
-        if (c0 + e < pr.p) mx[e] = max(mx[e], __float_as_uint(src[e]) & 0x7fffffffu);
+        if (k < pr.m && c0 + e < pr.p) mx[e] = max(mx[e], absb(pr.B[k * pr.p + c0 + e]));
     }
   }
 #pragma unroll
@@ -198,30 +210,40 @@ fp8blk_max_kernel(const SplitProb *__restrict__ probs, int nprobs) {
   }
 }
 
+// A quarter (blockIdx.y) of a pack tile: 32 rows of A or 64 columns of B by one
+// K block.  Bound by the loads in flight: quarters, and B's turn through shared
+// memory in 16-byte stores and whole pack rows written by eight lanes (entry (kk,
+// c) at column (c + 4 (kk / 16)) mod 64: those lanes' reads, 16 rows apart, then meet
+// no bank twice).  The tiles go last to first: the maxima pass read B last, so
+// most of it is still in L2.  4096^3, 168 MB: whole tiles, first to last, 62 us; now
+// 46.
+constexpr int kPackQuarters = 4;
+
 __global__ void __launch_bounds__(256)
 fp8blk_pack_kernel(const SplitProb *__restrict__ probs, int nprobs, const int *__restrict__ map,
                    uint32_t *__restrict__ pack) {
   constexpr int kQuads = kBK / 4;  // 32-bit words per pack row
-  __shared__ float tile[kBK][64 + 1];
-  __shared__ int colexp[64];
-  __shared__ uint32_t colmax[4][64];
-  const int item = blockIdx.x;
+  constexpr int kCols = kPackBN / kPackQuarters, kRows = kTcBM / kPackQuarters;
+  __shared__ __align__(16) float tile[kBK][kCols];
+  __shared__ int colexp[kCols];
+  __shared__ uint32_t colmax[8][kCols];
+  const int item = gridDim.x - 1 - blockIdx.x;
   const int g =
       find_problem(probs, nprobs, map, item, [](const SplitProb &q) { return q.pack_start; });
   const SplitProb &pr = probs[g];
   const int local = item - pr.pack_start;
-  const int tid = threadIdx.x, lane = tid & 31;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   if (local < pr.mt * pr.kt) {
-    // A tile (mt, kb): rows mt*128 + tid/32 + 8 it, a warp per row, four
+    // A tile (mt, kb): rows mt*128 + 32 y + warp + 8 it, a warp per row, four
     // values per lane
     const int mt = local / pr.kt, kb = local % pr.kt;
     const int64_t base = pr.a_row0 + (int64_t)local * kTcBM;
     const bool vec = al16(pr.A) && (pr.m & 3) == 0;
-    float4 xs[16];
+    const int r0 = (int)blockIdx.y * kRows + warp;
+    float4 xs[kRows / 8];
 #pragma unroll
-    for (int it = 0; it < 16; it++) {
-      const int r = (tid >> 5) + 8 * it;
-      const int64_t i = (int64_t)mt * kTcBM + r;
+    for (int it = 0; it < kRows / 8; it++) {
+      const int64_t i = (int64_t)mt * kTcBM + r0 + 8 * it;
       const int64_t k = (int64_t)kb * kBK + 4 * lane;
       float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
       if (i < pr.n) {
@@ -238,88 +260,82 @@ fp8blk_pack_kernel(const SplitProb *__restrict__ probs, int nprobs, const int *_
       xs[it] = x;
     }
 #pragma unroll
-    for (int it = 0; it < 16; it++) {
-      const int r = (tid >> 5) + 8 * it;
-      uint32_t mx = max(max(absb(xs[it].x), absb(xs[it].y)), max(absb(xs[it].z), absb(xs[it].w)));
+    for (int it = 0; it < kRows / 8; it++) {
+      const int r = r0 + 8 * it;
+      uint32_t mx = absmax4(xs[it]);
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
       const int e = pick_exponent(mx, pr.sA[(int64_t)mt * kTcBM + r]);
       if (lane == 0) fac_a(pr)[(int64_t)kb * pr.mt * kTcBM + (int64_t)mt * kTcBM + r] = pow2f(e);
       pack[(base + r) * kQuads + lane] = to_e4m3x4(xs[it], e);
     }
-  } else {
-    // B tile (nt, kb): 256 columns x 128 k, transposed through shared memory
-    // 64 columns at a time; one exponent per column of the block
-    const int b = local - pr.mt * pr.kt;
-    const int nt = b / pr.kt, kb = b % pr.kt;
-    const int64_t base = pr.b_row0 + (int64_t)b * kPackBN;
-    const bool vec = al16(pr.B) && (pr.p & 3) == 0;
-    for (int c0 = 0; c0 < kPackBN; c0 += 64) {
-      float4 vs[8];
+    return;
+  }
+  // B tile (nt, kb): columns 64 y + [0, 64) of 256 by 128 k, turned through shared
+  // memory; one exponent per column of the block
+  const int b = local - pr.mt * pr.kt;
+  const int nt = b / pr.kt, kb = b % pr.kt, c0 = (int)blockIdx.y * kCols;
+  const int64_t base = pr.b_row0 + (int64_t)b * kPackBN;
+  const bool vec = al16(pr.B) && (pr.p & 3) == 0;
+  const int c4 = tid % 16;  // vector of four columns, K rows tid / 16 + 16 it
+  const int64_t j = (int64_t)nt * kPackBN + c0 + 4 * c4;
+  float4 vs[8];
 #pragma unroll
-      for (int it = 0; it < 8; it++) {
-        const int q = tid + it * 256;  // 128 k rows x 16 vectors of 4 columns
-        const int kk = q / 16, c4 = q % 16;
-        const int64_t k = (int64_t)kb * kBK + kk;
-        const int64_t j = (int64_t)nt * kPackBN + c0 + 4 * c4;
-        float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (k < pr.m) {
-          const float *src = pr.B + k * pr.p + j;
-          if (vec && j + 4 <= pr.p) {
-            v = __ldcs(reinterpret_cast<const float4 *>(src));
-          } else {
-            if (j < pr.p) v.x = src[0];
-            if (j + 1 < pr.p) v.y = src[1];
-            if (j + 2 < pr.p) v.z = src[2];
-            if (j + 3 < pr.p) v.w = src[3];
-          }
-        }
-        vs[it] = v;
+  for (int it = 0; it < 8; it++) {
+    const int64_t k = (int64_t)kb * kBK + tid / 16 + 16 * it;
+    float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (k < pr.m) {
+      const float *src = pr.B + k * pr.p + j;
+      if (vec && j + 4 <= pr.p) {
+        v = __ldcs(reinterpret_cast<const float4 *>(src));
+      } else {
+        if (j < pr.p) v.x = src[0];
+        if (j + 1 < pr.p) v.y = src[1];
+        if (j + 2 < pr.p) v.z = src[2];
+        if (j + 3 < pr.p) v.w = src[3];
       }
-#pragma unroll
-      for (int it = 0; it < 8; it++) {
-        const int q = tid + it * 256;
-        const int kk = q / 16, c4 = q % 16;
-        tile[kk][4 * c4 + 0] = vs[it].x;
-        tile[kk][4 * c4 + 1] = vs[it].y;
-        tile[kk][4 * c4 + 2] = vs[it].z;
-        tile[kk][4 * c4 + 3] = vs[it].w;
-      }
-      __syncthreads();
-      {
-        // column maxima: four threads a column, 32 K values each
-        const int c = tid & 63, q = tid >> 6;
-        uint32_t mx = 0;
-#pragma unroll 8
-        for (int kk = 32 * q; kk < 32 * q + 32; kk++) mx = max(mx, absb(tile[kk][c]));
-        colmax[q][c] = mx;
-      }
-      __syncthreads();
-      if (tid < 64) {
-        const uint32_t mx = max(max(colmax[0][tid], colmax[1][tid]), max(colmax[2][tid], colmax[3][tid]));
-        const int e = pick_exponent(mx, pr.tB[(int64_t)nt * kPackBN + c0 + tid]);
-        colexp[tid] = e;
-        fac_b(pr)[(int64_t)kb * pr.nt * kPackBN + (int64_t)nt * kPackBN + c0 + tid] = pow2f(e);
-      }
-      __syncthreads();
-      for (int q = tid; q < 64 * (kBK / 16); q += 256) {
-        const int c = q % 64, k16 = q / 64;
-        const int e = colexp[c];
-        uint4 w;
-        uint32_t *wp = reinterpret_cast<uint32_t *>(&w);
-#pragma unroll
-        for (int t = 0; t < 4; t++) {
-          const int r = 16 * k16 + 4 * t;
-          wp[t] = to_e4m3x4(make_float4(tile[r][c], tile[r + 1][c], tile[r + 2][c], tile[r + 3][c]),
-                            e);
-        }
-        *reinterpret_cast<uint4 *>(pack + (base + c0 + c) * kQuads + 4 * k16) = w;
-      }
-      __syncthreads();
     }
+    vs[it] = v;
+  }
+  uint32_t mx[4] = {0, 0, 0, 0};
+#pragma unroll
+  for (int it = 0; it < 8; it++) {
+    *reinterpret_cast<float4 *>(&tile[tid / 16 + 16 * it][(4 * c4 + 4 * it) & (kCols - 1)]) = vs[it];
+    mx[0] = max(mx[0], absb(vs[it].x));
+    mx[1] = max(mx[1], absb(vs[it].y));
+    mx[2] = max(mx[2], absb(vs[it].z));
+    mx[3] = max(mx[3], absb(vs[it].w));
+  }
+#pragma unroll
+  for (int e = 0; e < 4; e++) {
+    mx[e] = max(mx[e], __shfl_xor_sync(0xffffffffu, mx[e], 16));  // the warp's two K rows
+    if (lane < 16) colmax[warp][4 * c4 + e] = mx[e];
+  }
+  __syncthreads();
+  if (tid < kCols) {
+    uint32_t m = 0;
+#pragma unroll
+    for (int w = 0; w < 8; w++) m = max(m, colmax[w][tid]);
+    const int e = pick_exponent(m, pr.tB[(int64_t)nt * kPackBN + c0 + tid]);
+    colexp[tid] = e;
+    fac_b(pr)[(int64_t)kb * pr.nt * kPackBN + (int64_t)nt * kPackBN + c0 + tid] = pow2f(e);
+  }
+  __syncthreads();
+#pragma unroll
+  for (int q = tid; q < kCols * (kBK / 16); q += 256) {
+    const int c = q / 8, k16 = q % 8;  // eight lanes a pack row
+    const int e = colexp[c];
+    const float *t = &tile[16 * k16][(c + 4 * k16) & (kCols - 1)];
+    uint4 w;
+    uint32_t *wp = reinterpret_cast<uint32_t *>(&w);
+#pragma unroll
+    for (int r = 0; r < 4; r++)
+      wp[r] = to_e4m3x4(make_float4(t[(4 * r) * kCols], t[(4 * r + 1) * kCols], t[(4 * r + 2) * kCols],
+                                    t[(4 * r + 3) * kCols]),
+                        e);
+    *reinterpret_cast<uint4 *>(pack + (base + c0 + c) * kQuads + 4 * k16) = w;
   }
 }
-
 
 // Tiles whose exponents do not change along K.  For row tile mt of A (items
 // [0, mt) of a problem) or column tile nt of B (items [mt, mt + nt)), flag 1
@@ -329,8 +345,10 @@ fp8blk_pack_kernel(const SplitProb *__restrict__ probs, int nprobs, const int *_
 // accumulated in tensor memory and the factor 2^(e_i + e_j), the same for
 // every block, is applied once; elsewhere each block is unscaled on its own.
 // flags: the problem's `cnt` array, mt + nt words; item prefix `ver_start`.
+// *any is set where a flag is 0: without one the blockwise kernel has no tiles.
 __global__ void __launch_bounds__(128)
-fp8blk_flag_kernel(const SplitProb *__restrict__ probs, int nprobs) {
+fp8blk_flag_kernel(const SplitProb *__restrict__ probs, int nprobs, int *any) {
+  pdl_wait();
   const int item = blockIdx.x;
   const int g =
       find_problem(probs, nprobs, nullptr, item, [](const SplitProb &q) { return q.ver_start; });
@@ -346,7 +364,10 @@ fp8blk_flag_kernel(const SplitProb *__restrict__ probs, int nprobs) {
   bool same = __uint_as_float(whole) <= 3.402823466e38f;
   for (int kb = 1; kb < pr.kt; kb++) same &= f[(int64_t)kb * width] == f0;
   same = __syncthreads_and(same);
-  if (threadIdx.x == 0) pr.cnt[local] = same ? 1 : 0;
+  if (threadIdx.x == 0) {
+    pr.cnt[local] = same ? 1 : 0;
+    if (!same) atomicOr(any, 1);
+  }
 }
 
 __device__ __forceinline__ bool tile_uniform(const SplitProb &pr, int mt, int nt) {
@@ -378,7 +399,11 @@ __device__ __forceinline__ void blk_unit(const SplitProb *__restrict__ probs, in
 
 __global__ void __launch_bounds__(kThreads, 1)
 fp8blk_gemm_kernel(const __grid_constant__ CUtensorMap tmap, const SplitProb *__restrict__ probs,
-                   int nprobs, const int *__restrict__ unit_map, int total_units, int *err) {
+                   int nprobs, const int *__restrict__ unit_map, int total_units, const int *any, int *err) {
+  // every tile keeps its factors along K: nothing to do (an empty pass over
+  // the tiles takes 10 us at 4096^3)
+  pdl_wait();
+  if (*reinterpret_cast<const volatile int *>(any) == 0) return;
   extern __shared__ uint8_t smem_raw[];
   const uint32_t raw = smem_u32(smem_raw);
   const uint32_t sbase = (raw + 1023u) & ~1023u;
@@ -667,7 +692,8 @@ mm_status fp8_blocks_launch(Scratch &ws, std::vector<SplitProb> &blk, std::vecto
   const size_t pack_bytes = (size_t)rows * kPackRowBytes;
   const size_t exp_off = (pack_bytes + 255) & ~(size_t)255;
   const size_t max_off = (exp_off + (size_t)exps * 4 + 255) & ~(size_t)255;
-  const size_t flag_off = (max_off + (size_t)maxw * 4 + 255) & ~(size_t)255;
+  const size_t any_off = max_off + (size_t)maxw * 4;  // zeroed with the maxima
+  const size_t flag_off = (any_off + 4 + 255) & ~(size_t)255;
   const size_t tab_off = (flag_off + (size_t)flag_items * 4 + 255) & ~(size_t)255;
   const size_t tab_bytes = (size_t)np * sizeof(SplitProb);
   const size_t map_off = (tab_off + 2 * tab_bytes + 255) & ~(size_t)255;
@@ -687,6 +713,7 @@ mm_status fp8_blocks_launch(Scratch &ws, std::vector<SplitProb> &blk, std::vecto
   }
   SplitProb *d_blk = reinterpret_cast<SplitProb *>(base + tab_off);
   SplitProb *d_tc = d_blk + np;
+  int *any = reinterpret_cast<int *>(base + any_off);
   {
     std::vector<uint8_t> blob(2 * tab_bytes, 0);
     std::memcpy(blob.data(), blk.data(), tab_bytes);
@@ -694,7 +721,7 @@ mm_status fp8_blocks_launch(Scratch &ws, std::vector<SplitProb> &blk, std::vecto
     e = ws.stage.copy_to_device(d_blk, blob.data(), blob.size(), s);
   }
   // whole-row and whole-column maxima first (zeroed: columns merge by atomicMax)
-  if (e == cudaSuccess) e = cudaMemsetAsync(base + max_off, 0, (size_t)maxw * 4, s);
+  if (e == cudaSuccess) e = cudaMemsetAsync(base + max_off, 0, (size_t)maxw * 4 + 4, s);
   if (e != cudaSuccess) return note_cuda(e);
   {
     TraceScope ts("fp8_max", s);
@@ -712,11 +739,11 @@ mm_status fp8_blocks_launch(Scratch &ws, std::vector<SplitProb> &blk, std::vecto
   }
   {
     TraceScope ts("fp8_pack", s);
-    fp8blk_pack_kernel<<<(unsigned)packs, 256, 0, s>>>(d_tc, np, pack_map,
+    fp8blk_pack_kernel<<<dim3((unsigned)packs, kPackQuarters), 256, 0, s>>>(d_tc, np, pack_map,
                                                        static_cast<uint32_t *>(ws.ptr));
     if ((e = cudaGetLastError()) != cudaSuccess) return note_cuda(e);
-    fp8blk_flag_kernel<<<(unsigned)flag_items, 128, 0, s>>>(d_blk, np);
-    if ((e = cudaGetLastError()) != cudaSuccess) return note_cuda(e);
+    e = launch_pdl_if(true, fp8blk_flag_kernel, (unsigned)flag_items, 128, 0, s, (const SplitProb *)d_blk, np, any);
+    if (e != cudaSuccess) return note_cuda(e);
   }
   // the uniform 128 x 256 tiles: one factor per row and column
   TcConfig cfg{128, 4, 0};
@@ -736,9 +763,9 @@ mm_status fp8_blocks_launch(Scratch &ws, std::vector<SplitProb> &blk, std::vecto
   if ((e = blk_pack_map(&map, ws.ptr, rows)) != cudaSuccess) return note_cuda(e);
   const int grid = (int)std::min<int64_t>(blk_units, sm_count());
   TraceScope ts("fp8_blk", s);
-  fp8blk_gemm_kernel<<<grid, kThreads, Lay::kSmem, s>>>(map, d_blk, np, blk_map, (int)blk_units,
-                                                        g_ctx.d_err);
-  return note_cuda(cudaGetLastError());
+  return note_cuda(launch_pdl_if(true, fp8blk_gemm_kernel, (unsigned)grid, kThreads, Lay::kSmem, s, map,
+                                 (const SplitProb *)d_blk, np, (const int *)blk_map, (int)blk_units,
+                                 (const int *)any, g_ctx.d_err));
 }
 
 }  // namespace
