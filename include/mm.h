@@ -48,6 +48,10 @@
  *                         2^-21) where the operands' magnitudes fit fp16, and
  *                         takes this form where they do not (a device-side
  *                         choice from the data).  Not in the paper.
+ *                         In both split modes the smallest products that
+ *                         mm_gemm would give the fused kernel (a few
+ *                         microseconds of multiply-adds) run as MM_MODE_SIMT,
+ *                         which is faster and more accurate there.
  *   MM_MODE_AUTO          SPLIT_BF16X3 for MM_F32, DGEMM for MM_F64.
  *   MM_MODE_OZAKI         FP64 in/out on the e4m3 tensor cores (Ozaki
  *                         scheme): each row of A / column of B is scaled by a

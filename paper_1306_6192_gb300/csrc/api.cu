@@ -333,6 +333,11 @@ mm_status enqueue_gemm(int64_t n, int64_t m, int64_t p, const void *A, const voi
       const FusedPlan fpl = fused_plan(n, m, p, kind);
       const bool fused = fpl.S > 0 && fused_operands_ok(static_cast<const float *>(A),
                                                         static_cast<const float *>(B), m, p);
+      if (fused) {
+        // the smallest ones: FP32 multiply-adds, exact terms in one or two short launches
+        const SimtPlan spl = simt_plan(false, n, m, p);
+        if (simt_beats_fused(n, m, p, spl)) return enqueue_gemm(n, m, p, A, B, C, dt, MM_MODE_SIMT, s, epi);
+      }
       // with m < 2237 and more than three K blocks a slice the packed fp16 form is
       // faster: the fused kernel converts every operand for each of its tiles
       // (GB300, fused against packed: 512^3 at one block 17 / 19 us, 300 x 2236 x

@@ -217,6 +217,14 @@ struct SimtPlan {
 SimtPlan simt_plan(bool f64, int64_t n, int64_t m, int64_t p);
 // The same plan for a device of `sms` SMs (host only; mm_simt_plan).
 SimtPlan simt_plan_for(bool f64, int64_t n, int64_t m, int64_t p, int sms);
+// Whether an FP32 product that the fused tensor-core kernel would take runs on
+// the CUDA cores instead: the multiply-adds of the busiest SM, in cycles, against
+// the fused kernel's start-up and exchange.  GB300, us fused / SIMT: 64 x 512 x 64
+// 9.6 / 4.8, 256^3 11.6 / 5.2, 128 x 4096 x 128 15.9 / 8.9 (4096 cycles), 64 x 16384 x 64 19.2 /
+// 10.0; 256 x 4096 x 256 (14336) 22.9 / 20.0, 768^3 22.1 / 26.5, 512 x 2048 x 512 28.5 /
+// 36.5 stay with the tensor cores.  In a cluster the line is lower (512^3, 7168 cycles, 17.1 / 11.5, stays): products of
+// that size are documented as one launch of the fused kernel.
+bool simt_beats_fused(int64_t n, int64_t m, int64_t p, const SimtPlan &pl);
 size_t simt_scratch_bytes(bool f64, int64_t n, int64_t m, int64_t p);
 cudaError_t launch_simt_splitk_f32(int64_t n, int64_t m, int64_t p, const float *A, const float *B,
                                    float *C, float *part, const SimtPlan &pl, cudaStream_t s,

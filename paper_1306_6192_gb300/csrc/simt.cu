@@ -650,6 +650,13 @@ size_t simt_scratch_bytes(bool f64, int64_t n, int64_t m, int64_t p) {
   return pl.S > 1 ? (size_t)pl.S * (size_t)(n * p) * (f64 ? 8 : 4) : 0;
 }
 
+bool simt_beats_fused(int64_t n, int64_t m, int64_t p, const SimtPlan &pl) {
+  if (pl.S < 1) return false;
+  const int64_t rounds = ceil_div(ceil_div(n, 32) * ceil_div(p, 32) * pl.S, (int64_t)sm_count());
+  const int64_t cycles = rounds * 1024 * pl.ks / 128;
+  return cycles <= (pl.S <= kSimtCluster ? 6144 : 8192);
+}
+
 cudaError_t launch_simt_splitk_f32(int64_t n, int64_t m, int64_t p, const float *A, const float *B,
                                    float *C, float *part, const SimtPlan &pl, cudaStream_t s,
                                    const Epi *epi) {
