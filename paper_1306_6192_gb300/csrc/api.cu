@@ -338,12 +338,15 @@ mm_status enqueue_gemm(int64_t n, int64_t m, int64_t p, const void *A, const voi
         const SimtPlan spl = simt_plan(false, n, m, p);
         if (simt_beats_fused(n, m, p, spl)) return enqueue_gemm(n, m, p, A, B, C, dt, MM_MODE_SIMT, s, epi);
       }
-      // with m < 2237 and more than three K blocks a slice the packed fp16 form is
-      // faster: the fused kernel converts every operand for each of its tiles
-      // (GB300, fused against packed: 512^3 at one block 17 / 19 us, 300 x 2236 x
-      // 300 at three 26 / 29, 1024 x 1024 x 512 at four 26 / 24.5, 1024^3 at eight
-      // 44.5 / 25.1)
-      if (fused && (kind != kTcSplitF16x3 || ceil_div(ceil_div(m, 64), fpl.S) <= 3)) {
+      // with m < 2237 the packed form takes long slices: the fused kernel converts
+      // every operand for each of its tiles, about 9 + 4.4 us a K block of a slice.
+      // The data may turn the packed form to six products (magnitudes out of
+      // fp16's range), about 30 + 0.9 us a K block of the whole, so the line lies
+      // where that is no slower.  GB300, us fused / packed / packed with six:
+      // 1024^3 at eight blocks 44.5 / 25.1 / 44.8; 640 x 1280 x 768 39.9 / - / 50.0 and
+      // 512 x 1100 x 900 30.9 / - / 47.2 stay.
+      const int64_t kb = ceil_div(m, 64), slice = fused ? ceil_div(kb, fpl.S) : 0;
+      if (fused && (kind != kTcSplitF16x3 || 44 * slice < 205 + 9 * kb)) {
         return run_fused(g_ctx.fused_ws, n, m, p, static_cast<const float *>(A),
                          static_cast<const float *>(B), static_cast<float *>(C), kind, fpl, s, epi);
       }

@@ -60,6 +60,7 @@
 
 #include <algorithm>
 
+#include "ctx.h"
 #include "tc_ptx.cuh"
 #include "tc_units.cuh"
 
@@ -261,7 +262,7 @@ tc_half_kernel(const __grid_constant__ CUtensorMap map, const __grid_constant__ 
           if (k1 < 0) break;
           uint32_t t0 = 0;
           for (int ki = k0; ki < k1; ki++) {
-            const bool first = ki == k0 || (!x6 && ((ki - k0) & in_chunk) == 0);
+            const bool first = ((ki - k0) & in_chunk) == 0;
             if (first) {
               // the accumulator of the last chunk goes to the epilogue
               if (ki != k0) {
@@ -355,7 +356,10 @@ tc_half_kernel(const __grid_constant__ CUtensorMap map, const __grid_constant__ 
           d.sA = pr.sA;
           d.tB = pr.tB;
           d.split_s = pr.split_s;
-          d.chunk = pr.chunk;
+          // three parts, in stages of 32 K: one sum over K, as tc_gemm.cu's, or every
+          // 64 K for products that the fused kernel served (magnitudes over many
+          // binades, 1024^3: error 3.7e-6 in one sum, 2.6e-7 in the fused kernel's)
+          d.chunk = !x6 ? pr.chunk : (pr.chunk < kHalfChunk ? 2 : 1 << 30);
           d.h = tc.h;
           const int st = tc.t - pr.split_from;
           d.part = tc.h >= 0 ? pr.part + (size_t)st * pr.split_s * (kTcBM * kBN) : nullptr;
@@ -412,7 +416,7 @@ tc_half_kernel(const __grid_constant__ CUtensorMap map, const __grid_constant__ 
       if (d->k1 < 0) break;
       const int n = d->n, p = d->p, x6 = d->x6, h = d->h, split_s = d->split_s, epi_on = d->epi_on;
       const int row0 = d->row0 + q * 32, col0 = d->col0;
-      const int chunks = x6 ? 1 : (d->k1 - d->k0 + d->chunk - 1) / d->chunk;
+      const int chunks = (d->k1 - d->k0 + d->chunk - 1) / d->chunk;
       // whole 32-byte sectors: C (and D) 32-byte aligned, p % 8 == 0
       const bool vec8 = d->vec8 != 0;
       const bool vec_d = vec8 && epi_on == 2;

@@ -94,3 +94,23 @@ def test_split_tail_and_epilogue(mmlib, p):
     e, _ = full_errors(C.cpu().numpy(), A, B)
     assert e.max() <= oracle.tolerance(m, "f32")
     assert torch.equal(E, C - dD)
+
+
+@pytest.mark.parametrize("shape", [(1024, 1024, 1024), (640, 1280, 768)], ids=lambda s: "x".join(map(str, s)))
+def test_wide_products_keep_short_sums(mmlib, shape):
+    """Magnitudes over 40 binades take three bf16 parts; products that the fused
+    kernel's plan covers add them every 64 K, so that a sum's error stays that of
+    m / 64 roundings to nearest and of 24 truncations within a block: 2^-24
+    (sqrt(m / 64) + 24 / sqrt(m / 64)) of the result's norm, doubled here (one sum
+    over K loses 3.7e-6)."""
+    n, m, p = shape
+    g = torch.Generator(device="cuda").manual_seed(77)
+    spread = lambda r, c: (torch.rand(r, c, device="cuda", generator=g) * 2 - 1) * torch.exp2(
+        torch.randint(-20, 21, (r, c), device="cuda", generator=g).float())
+    A, B = spread(n, m), spread(m, p)
+    C = torch.empty(n, p, device="cuda")
+    assert mmlib.mm_tune_query_splitk(n, m, p)[2] > 0
+    assert mmlib.mm_gemm(n, m, p, A, B, C, mmlib.MM_F32, mmlib.MM_MODE_SPLIT_BF16X3) == mmlib.MM_OK
+    E = A.double() @ B.double()
+    b = (m / 64) ** 0.5
+    assert ((C.double() - E).norm() / E.norm()).item() <= 2 * 2.0 ** -24 * (b + 24 / b)
