@@ -44,10 +44,12 @@
  *                         For inner dimensions m < 2237, where two bf16 parts
  *                         cannot meet its tolerance, SPLIT_BF16X3 itself splits
  *                         every operand, scaled by one power of two, into two
- *                         fp16 parts (three products, each term within about
- *                         2^-21) where the operands' magnitudes fit fp16, and
- *                         takes this form where they do not (a device-side
- *                         choice from the data).  Not in the paper.
+ *                         fp16 parts (three products, each term within
+ *                         3 * 2^-22, or for m >= 64 and factors about 2^-28 of
+ *                         their operand's largest entries 2^-17.4) where the
+ *                         operands' magnitudes fit fp16 and m > 16, and takes
+ *                         this form elsewhere (a device-side choice from the
+ *                         data).  Not in the paper.
  *                         In both split modes the smallest products that
  *                         mm_gemm would give the fused kernel (a few
  *                         microseconds of multiply-adds) run as MM_MODE_SIMT,

@@ -112,9 +112,10 @@ mm_status note_cuda(cudaError_t e);
 
 // Kind of split used for inner dimension m: two bf16 parts (three products)
 // where their worst-case per-product error 3 * 2^-16 is within the stated
-// tolerance 1e-6 sqrt(m); below that two fp16 parts (three products, at most
-// 2^-21 per product) where the magnitudes allow them, else three bf16 parts
-// (six products).
+// tolerance 1e-6 sqrt(m); below that two fp16 parts (three products, each
+// within 3 * 2^-22, or 2^-18 + 2^-19 in the lowest two binades of their window, which
+// only m >= 64 uses) where the magnitudes allow them and m > 16, else three bf16
+// parts (six products).
 TcKind split_kind_for(int64_t m);
 // The kind a split-path mode runs with for inner dimension m.
 inline TcKind split_kind_of(mm_mode mode, int64_t m) {

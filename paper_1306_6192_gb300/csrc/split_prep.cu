@@ -31,17 +31,29 @@
 // tolerance): x 2^e = hi + 2^-11 lo with hi = fp16_rn(x 2^e) and lo =
 // fp16_rn(2^11 (x 2^e - hi)), one e per operand of a product.  fp16 carries
 // eleven bits a part against bf16's eight, so two parts hold what three bf16
-// parts hold (|x 2^e - hi - 2^-11 lo| <= 2^-23 |x 2^e|) and three products
+// parts hold and three products
 // replace six; keeping lo scaled by 2^11 (R. Ootomo, R. Yokota, "Recovering
 // single precision accuracy from Tensor Cores while surpassing the FP32
 // theoretical peak performance", IJHPCA 36, 2022) keeps it out of fp16's
-// subnormals for |x 2^e| down to 2^-14.  e comes from a sample of the operand
-// (split_maps_kernel, or
-// the pack itself in a table of one product), the pack tests every entry against the window
-// [2^-16, 61440] of |x 2^e| (zeros pass; at 2^-16 the two parts are within
-// 2^-20 of the entry), and a product with an entry outside is packed
+// subnormals.  e comes from a sample of the operand (split_maps_kernel, or
+// the pack itself in a table of one product), the pack tests every entry against
+// the window of |x 2^e| (zeros pass), and a product with an entry outside is packed
 // again by the fix pass as three bf16 parts, scaled where it must be; one
 // whose sample already spreads too far is packed so from the start.
+//
+// The window, by what the two parts lose.  |x 2^e| from 2^-14 to 61440: hi is a normal
+// fp16 number, hi + 2^-11 lo is within 2^-22 of the entry and lo within 2^-11 of
+// it, so a term of C (both operands, and the product of the two low parts, which is
+// dropped) is within 3 * 2^-22 = 7.2e-7.  Below, hi is a subnormal: at 2^-16 the
+// entry is within 2^-20 and lo reaches 2^-9 of it, so a term of two such entries
+// is off by up to 2^-18 + 2^-19 = 5.7e-6, all terms of an entry of C alike where a whole
+// row of A and column of B lie there.  The tolerance 1e-6 sqrt(m) covers that, with
+// 2.3e-6 left for the sums, from m = 64 on: the window starts at 2^-16 there, and at
+// 2^-14 below (2 more of the 29 binades under the largest sampled entry then turn a
+// product to three parts).  m <= 16 always takes three parts: K in one MMA of
+// sixteen leaves the sums nothing to lose, and the six products are the
+// more accurate ones (1000 x 16 x 1000, largest error over |A||B| 1.1e-7 against
+// 1.8e-7; m = 1 1.5e-7 against 4.6e-7; m = 24 4.5e-7 against 2.2e-7).
 #include <algorithm>
 
 #include <cuda_fp16.h>
@@ -52,12 +64,16 @@ namespace mm {
 namespace {
 
 // Window of |x 2^e| that the two fp16 parts take (its ends as FP32 bit
-// patterns), and the exponent that the largest
+// patterns; the lower one by the inner dimension), and the exponent that the largest
 // sampled magnitude is brought to (a factor of at least 3.75 of room above
-// it, 2^29 below).  kHalfExpMax bounds |e| so that 2^e, the window's ends
+// it, 2^29 or 2^27 below).  kHalfExpMax bounds |e| so that 2^e, the window's ends
 // divided by 2^e and the products stay normal FP32 numbers.
 constexpr int kHalfTopExp = 13, kHalfExpMax = 100;
-constexpr uint32_t kHalfLowBits = 0x37800000u, kHalfHighBits = 0x47700000u;  // 2^-16, 61440
+constexpr uint32_t kHalfHighBits = 0x47700000u;  // 61440
+constexpr int kHalfMinK = 17;                    // fewer K values take three parts
+__device__ __forceinline__ uint32_t half_low_bits(int m) {
+  return m >= 64 ? 0x37800000u : 0x38800000u;  // 2^-16, 2^-14
+}
 constexpr int kHalfSamples = 256;  // entries sampled per operand
 
 __device__ __forceinline__ uint32_t abs_bits(float x) { return __float_as_uint(x) & 0x7fffffffu; }
@@ -120,11 +136,11 @@ __device__ __forceinline__ uint32_t min4_bits(float4 x) {
   return min(a, min(abs_bits(x.z) - 1u, abs_bits(x.w) - 1u));
 }
 
-// An operand with an entry outside the fp16 window: |x| in [2^-16, 61440]
+// An operand with an entry outside the fp16 window [low, 61440]
 // times 2^-e, as bit patterns (both ends are normal numbers for |e| <= 100).
-__device__ __forceinline__ bool outside_window(uint32_t mx, uint32_t mn, int e) {
+__device__ __forceinline__ bool outside_window(uint32_t mx, uint32_t mn, int e, uint32_t low) {
   const uint32_t shift = (uint32_t)e << 23;
-  return mx > kHalfHighBits - shift || mn < kHalfLowBits - shift - 1u;
+  return mx > kHalfHighBits - shift || mn < low - shift - 1u;
 }
 
 // max |x| over four values as a float bit pattern
@@ -365,12 +381,20 @@ __device__ __forceinline__ uint2 sample_range(const float *__restrict__ X, int64
 
 // The fp16 window's exponent e for an operand of that range: its largest
 // sampled magnitude to [2^13, 2^14).  False where the sample does not fit.
-__device__ __forceinline__ bool half_exponent(uint2 range, int &e) {
+__device__ __forceinline__ bool half_exponent(uint2 range, uint32_t low, int &e) {
   e = 0;
   if (range.x == 0) return true;  // nothing but zeros sampled
   if (range.x >= 0x7f800000u) return false;
   e = kHalfTopExp - ilogbf(__uint_as_float(range.x));
-  return abs(e) <= kHalfExpMax && !outside_window(range.x, range.y, e);
+  return abs(e) <= kHalfExpMax && !outside_window(range.x, range.y, e, low);
+}
+
+// The form of a product from its operands' samples: 1 for three bf16 parts, 0
+// for two fp16 parts with the exponents ea and eb.
+__device__ __forceinline__ int half_form(uint2 ra, uint2 rb, int m, int &ea, int &eb) {
+  const uint32_t low = half_low_bits(m);
+  const bool fits = half_exponent(ra, low, ea) & half_exponent(rb, low, eb);
+  return fits && m >= kHalfMinK ? 0 : 1;
 }
 
 // The same for kTcSplitF16x3 tables (bn = 128): a product's tiles as two fp16
@@ -400,6 +424,7 @@ struct __align__(16) PackItem {
   int32_t ld;         // entries between its rows (A) / K rows (B)
   int32_t outer, k;   // rows (columns) and K values from its first entry to the edge
   int32_t e;          // exponent of the fp16 parts
+  uint32_t low;       // lower end of their window
   uint8_t is_a, x6, vec, pad;
 };
 constexpr int kPkStages = 3, kPkItems = 64;
@@ -482,7 +507,7 @@ __device__ __forceinline__ bool emit_tile(const PackItem &d, const float4 *t4, i
   const uint32_t mx = half_warp_max8(mxv);
   const int r = r0 + 16 * ((tid >> 1) & 7);
   if ((tid & 1) == 0 && r < d.outer) d.maxima[r] = mx;
-  return HALF && outside_window(mx, mn, d.e);
+  return HALF && outside_window(mx, mn, d.e, d.low);
 }
 
 __global__ void __launch_bounds__(288, 2)
@@ -500,7 +525,7 @@ split_pack_half_kernel(const __grid_constant__ ProbTable tab, const int *__restr
     int ea, eb;
     const uint2 ra = sample_range(probs->A, (int64_t)probs->n * probs->m, mx_s, mn_s);
     const uint2 rb = sample_range(probs->B, (int64_t)probs->m * probs->p, mx_s, mn_s);
-    const int x6 = (half_exponent(ra, ea) & half_exponent(rb, eb)) ? 0 : 1;
+    const int x6 = half_form(ra, rb, probs->m, ea, eb);
     if (tid == 0) {
       one[kHalfX6] = x6;
       one[kHalfExpA] = ea;
@@ -526,6 +551,7 @@ split_pack_half_kernel(const __grid_constant__ ProbTable tab, const int *__restr
       d.is_a = b < 0;
       d.x6 = hx[kHalfX6] != 0;
       d.e = hx[b < 0 ? kHalfExpA : kHalfExpB];
+      d.low = half_low_bits(pr.m);
       d.bad = &pr.hx[kHalfBad];
       const int t = b < 0 ? local : b;
       const int o0 = (t / pr.kt) * 128, kb = t % pr.kt;  // first row or column, K block
@@ -695,8 +721,7 @@ split_maps_kernel(const __grid_constant__ ProbTable tab, int *__restrict__ unit_
     const uint2 rb = sample_range(pr.B, (int64_t)pr.m * pr.p, mx_s, mn_s);
     if (threadIdx.x == 0) {
       int ea = 0, eb = 0;
-      const bool ok = half_exponent(ra, ea) & half_exponent(rb, eb);
-      pr.hx[kHalfX6] = ok ? 0 : 1;
+      pr.hx[kHalfX6] = half_form(ra, rb, pr.m, ea, eb);
       pr.hx[kHalfExpA] = ea;
       pr.hx[kHalfExpB] = eb;
     }

@@ -2,8 +2,8 @@
 // dimensions): C = A.B from two fp16 parts per operand (split_prep.cu)
 //     C_ij = 2^-(ea + eb) (sum_r (Ah Bh)_irj + 2^-11 sum_r (Ah Bl + Al Bh)_irj)
 // with Bl, Al the parts scaled by 2^11; the products of the two low parts,
-// below 2^-22 relative, are dropped.  A product whose magnitudes do not fit
-// fp16 was packed as three bf16 parts and runs here as the six products of
+// below 2^-22 of a term (2^-18 at the window's low end, split_prep.cu), are dropped.
+// A product whose magnitudes do not fit fp16, or with m <= 16, was packed as three bf16 parts and runs here as the six products of
 // tc_gemm.cu's three-part kind (hx, SplitProb): one launch serves both.
 //
 // Why this form.  Six bf16 products were the bound of every product with a
