@@ -53,7 +53,9 @@
  *                         In both split modes the smallest products that
  *                         mm_gemm would give the fused kernel (a few
  *                         microseconds of multiply-adds) run as MM_MODE_SIMT,
- *                         which is faster and more accurate there.
+ *                         which is faster and more accurate there; an entry
+ *                         whose FP32 sum overflows on the way is then summed
+ *                         again from scaled operands.
  *   MM_MODE_AUTO          SPLIT_BF16X3 for MM_F32, DGEMM for MM_F64.
  *   MM_MODE_OZAKI         FP64 in/out on the e4m3 tensor cores (Ozaki
  *                         scheme): each row of A / column of B is scaled by a

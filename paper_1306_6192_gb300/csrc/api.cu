@@ -290,6 +290,22 @@ static mm_status product_then_epilogue(int64_t n, int64_t p, void *C, mm_dtype d
   return unit ? MM_OK : enqueue_scale(n * p, epi.alpha, C, C, dt, s);
 }
 
+// A product with few output tiles on the CUDA cores: K slices and a fixed-order sum.
+static mm_status enqueue_simt_slices(bool f64, int64_t n, int64_t m, int64_t p, const void *A, const void *B,
+                                     void *C, const SimtPlan &pl, cudaStream_t s, const Epi *epi,
+                                     bool keep_range) {
+  void *part = nullptr;
+  if (pl.S > 1) {
+    cudaError_t e = g_ctx.simt_ws.reserve(simt_scratch_bytes(f64, n, m, p), s);
+    if (e != cudaSuccess) return note_cuda(e);
+    part = g_ctx.simt_ws.ptr;
+  }
+  return note_cuda(f64 ? launch_simt_splitk_f64(n, m, p, (const double *)A, (const double *)B, (double *)C,
+                                                (double *)part, pl, s, nullptr, epi)
+                       : launch_simt_splitk_f32(n, m, p, (const float *)A, (const float *)B, (float *)C,
+                                                (float *)part, pl, s, epi, keep_range));
+}
+
 // Queues C = A.B (device pointers) on stream s.
 mm_status enqueue_gemm(int64_t n, int64_t m, int64_t p, const void *A, const void *B, void *C,
                        mm_dtype dt, mm_mode mode, cudaStream_t s, const Epi *epi) {
@@ -304,22 +320,9 @@ mm_status enqueue_gemm(int64_t n, int64_t m, int64_t p, const void *A, const voi
   switch (md) {
     case MM_MODE_SIMT:
     case MM_MODE_DGEMM: {
-      // products with few output tiles: K slices and a fixed-order sum
       const bool f64 = md == MM_MODE_DGEMM;
       const SimtPlan pl = simt_plan(f64, n, m, p);
-      if (pl.S >= 1) {
-        void *part = nullptr;
-        if (pl.S > 1) {
-          cudaError_t e = g_ctx.simt_ws.reserve(simt_scratch_bytes(f64, n, m, p), s);
-          if (e != cudaSuccess) return note_cuda(e);
-          part = g_ctx.simt_ws.ptr;
-        }
-        return note_cuda(f64 ? launch_simt_splitk_f64(n, m, p, (const double *)A, (const double *)B,
-                                                      (double *)C, (double *)part, pl, s, nullptr,
-                                                      epi)
-                             : launch_simt_splitk_f32(n, m, p, (const float *)A, (const float *)B,
-                                                      (float *)C, (float *)part, pl, s, epi));
-      }
+      if (pl.S >= 1) return enqueue_simt_slices(f64, n, m, p, A, B, C, pl, s, epi, false);
       return note_cuda(f64 ? launch_simt_f64(n, m, p, (const double *)A, (const double *)B,
                                              (double *)C, s, nullptr, epi)
                            : launch_simt_f32(n, m, p, (const float *)A, (const float *)B,
@@ -336,7 +339,7 @@ mm_status enqueue_gemm(int64_t n, int64_t m, int64_t p, const void *A, const voi
       if (fused) {
         // the smallest ones: FP32 multiply-adds, exact terms in one or two short launches
         const SimtPlan spl = simt_plan(false, n, m, p);
-        if (simt_beats_fused(n, m, p, spl)) return enqueue_gemm(n, m, p, A, B, C, dt, MM_MODE_SIMT, s, epi);
+        if (simt_beats_fused(n, m, p, spl)) return enqueue_simt_slices(false, n, m, p, A, B, C, spl, s, epi, true);
       }
       // with m < 2237 the packed form takes long slices: the fused kernel converts
       // every operand for each of its tiles, about 9 + 4.4 us a K block of a slice.

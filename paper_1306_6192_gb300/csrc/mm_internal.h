@@ -226,9 +226,11 @@ SimtPlan simt_plan_for(bool f64, int64_t n, int64_t m, int64_t p, int sms);
 // that size are documented as one launch of the fused kernel.
 bool simt_beats_fused(int64_t n, int64_t m, int64_t p, const SimtPlan &pl);
 size_t simt_scratch_bytes(bool f64, int64_t n, int64_t m, int64_t p);
+// keep_range (products of the split modes): entries whose FP32 sum leaves the
+// range are summed again, scaled (simt.cu).
 cudaError_t launch_simt_splitk_f32(int64_t n, int64_t m, int64_t p, const float *A, const float *B,
                                    float *C, float *part, const SimtPlan &pl, cudaStream_t s,
-                                   const Epi *epi = nullptr);
+                                   const Epi *epi = nullptr, bool keep_range = false);
 // run_if: as for launch_simt_f64 (the FP64 emulation's fallback).
 cudaError_t launch_simt_splitk_f64(int64_t n, int64_t m, int64_t p, const double *A,
                                    const double *B, double *C, double *part, const SimtPlan &pl,

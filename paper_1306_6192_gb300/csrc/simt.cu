@@ -259,14 +259,48 @@ simt_splitk_kernel(const T *__restrict__ A, const T *__restrict__ B, OutPtr<T, E
                                             n, m, kb, p, blockIdx.y, blockIdx.x, epi);
 }
 
+// A product of a split mode keeps its entries finite where the terms cancel, as its
+// tensor-core kernels do by scaling: an entry whose FP32 sum left the range
+// (an infinity, or a NaN of two; a sum that stays finite never left it) is
+// summed again with A and B times 2^-72 each, r ascending.  An overflow means
+// (|A||B|)_ij >= 2^127, against which the bits that the factor costs entries
+// below 2^-54 (2^-78 of the other factor, below 2^50) are nothing.  Infinities
+// and NaNs of A or B themselves keep the sum v as it came out.  One thread an
+// entry, after the others are stored: slow (64 x 16384 x 64 with all of C so, 0.74 ms), but
+// other data pays only the test (9.90 us against 9.82).
+struct RangeArgs {
+  const float *A, *B;
+  int64_t m, p;
+};
+__device__ __forceinline__ float sum_in_range(float v, const RangeArgs &x, int64_t row, int64_t col) {
+  const float *a = x.A + row * x.m, *b = x.B + col;
+  float acc = 0.0f;
+#pragma unroll 1
+  for (int64_t r0 = 0; r0 < x.m; r0 += 8) {
+    float s[8], t[8];
+    bool finite = true;
+#pragma unroll
+    for (int e = 0; e < 8; e++) {
+      s[e] = r0 + e < x.m ? a[r0 + e] : 0.0f;
+      t[e] = r0 + e < x.m ? b[(r0 + e) * x.p] : 0.0f;
+      finite &= isfinite(s[e]) && isfinite(t[e]);
+    }
+    if (!finite) return v;
+#pragma unroll
+    for (int e = 0; e < 8; e++) acc = fmaf(s[e] * 0x1p-72f, t[e] * 0x1p-72f, acc);
+  }
+  return acc * 0x1p72f * 0x1p72f;
+}
+
 // C = sum over s of part[s] for the np entries, 32 consecutive entries per
 // block (the loads of a slice coalesce): warp g adds slices [g S / G,
 // (g + 1) S / G) in order (G = min(8, S)), then the G partial sums are added
 // in the order g = 0, 1, ..., G - 1; the epilogue epi is applied to the sum.
-template <typename T>
+// RANGE: sum_in_range's entries.
+template <typename T, bool RANGE = false>
 __global__ void __launch_bounds__(256)
 splitk_sum_kernel(const T *__restrict__ part, int S, int64_t np, T *C,
-                  const int *__restrict__ run_if, EpiT<T> epi) {
+                  const int *__restrict__ run_if, EpiT<T> epi, RangeArgs range) {
   __shared__ T ps[8][32];
   asm volatile("griddepcontrol.wait;" ::: "memory");  // the slices' partials are written
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
@@ -285,6 +319,8 @@ splitk_sum_kernel(const T *__restrict__ part, int S, int64_t np, T *C,
   if (g == 0 && i < np) {
     T acc = ps[0][lane];
     for (int gg = 1; gg < G; gg++) acc += ps[gg][lane];
+    if constexpr (RANGE)
+      if (!isfinite(acc)) acc = sum_in_range(acc, range, i / range.p, i % range.p);
     C[i] = epi_apply(epi, acc, i);
   }
 }
@@ -353,10 +389,24 @@ cudaError_t launch_dependent(void (*kernel)(KArgs...), dim3 grid, cudaStream_t s
   return cudaLaunchKernelEx(&cfg, kernel, args...);
 }
 
+// The sum of S slices' partials into C.
+template <typename T>
+cudaError_t launch_sum(int64_t n, int64_t m, int64_t p, const T *A, const T *B, T *C, const T *part, int S,
+                       cudaStream_t s, const int *run_if, const EpiT<T> &ep, bool keep_range) {
+  TraceScope ts("simt_sum", s);
+  const int64_t np = n * p;
+  if (ceil_div(np, 32) > 2147483647LL) return cudaErrorInvalidValue;
+  const dim3 grid((unsigned)ceil_div(np, 32), 1, 1);
+  if constexpr (std::is_same_v<T, float>)
+    if (keep_range)
+      return launch_dependent(splitk_sum_kernel<T, true>, grid, s, part, S, np, C, run_if, ep, RangeArgs{A, B, m, p});
+  return launch_dependent(splitk_sum_kernel<T>, grid, s, part, S, np, C, run_if, ep, RangeArgs{});
+}
+
 template <typename T, int BM, int BN, int BK, int TM, int TN>
 cudaError_t launch_splitk(int64_t n, int64_t m, int64_t p, const T *A, const T *B, T *C, T *part,
                           const SimtPlan &pl, cudaStream_t s, const char *name,
-                          const int *run_if, const Epi *epi) {
+                          const int *run_if, const Epi *epi, bool keep_range = false) {
   constexpr int W = 16 / (int)sizeof(T);
   const int64_t gy = ceil_div(n, BM), gx = ceil_div(p, BN);
   if (gy > 65535 || gx > 2147483647LL || pl.S < 1 || pl.S > 65535) return cudaErrorInvalidValue;
@@ -382,11 +432,7 @@ cudaError_t launch_splitk(int64_t n, int64_t m, int64_t p, const T *A, const T *
                                  n, m, p, pl.ks, run_if, slice_ep);
   }
   if (e != cudaSuccess || pl.S == 1) return e;
-  TraceScope ts("simt_sum", s);
-  const int64_t np = n * p;
-  if (ceil_div(np, 32) > 2147483647LL) return cudaErrorInvalidValue;
-  return launch_dependent(splitk_sum_kernel<T>, dim3((unsigned)ceil_div(np, 32), 1, 1), s,
-                          static_cast<const T *>(part), pl.S, np, C, run_if, ep);
+  return launch_sum(n, m, p, A, B, C, part, pl.S, s, run_if, ep, keep_range);
 }
 
 // Small FP32 tiles: BM x BN outputs, TM x 4 a thread, a warp 4 TM x 32.  The
@@ -425,7 +471,8 @@ __device__ __forceinline__ void copy_or_zero(uint32_t dst, const float *src, boo
   }
 }
 
-template <int BM, int BN, int TM, bool VEC, bool EPI>
+// RANGE: sum_in_range's entries (with `out` C itself).
+template <int BM, int BN, int TM, bool VEC, bool EPI, bool RANGE>
 __global__ void __launch_bounds__(RingShape<BM, BN, TM>::NT)
 simt_ring_kernel(const float *__restrict__ A, const float *__restrict__ B, OutPtr<float, EPI> out, int64_t n,
                  int64_t m, int64_t p, int64_t ks, int cluster, bool early, EpiT<float> epi) {
@@ -495,26 +542,47 @@ simt_ring_kernel(const float *__restrict__ A, const float *__restrict__ B, OutPt
 
   if (!early) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 
-  auto put = [&](float *C, int64_t row, int64_t col, float4 v, bool apply) {
-    if (row >= n || col >= p) return;
+  // Four entries of a row; with RANGE, returns those that are not finite (a bit
+  // each) and leaves them to put_again.
+  auto put = [&](float *C, int64_t row, int64_t col, float4 v) -> uint32_t {
+    if (row >= n || col >= p) return 0;
     const int64_t x = row * p + col;
     float t[4] = {v.x, v.y, v.z, v.w};
-    if (VEC) {
+    uint32_t left = 0;
+    if (RANGE) {
 #pragma unroll
-      for (int e = 0; e < 4; e++) t[e] = EPI && apply ? epi_apply(epi, t[e], x + e) : t[e];
+      for (int e = 0; e < 4; e++) left |= (uint32_t)((VEC || col + e < p) && !isfinite(t[e])) << e;
+    }
+    if (VEC && left == 0) {
+#pragma unroll
+      for (int e = 0; e < 4; e++) t[e] = EPI ? epi_apply(epi, t[e], x + e) : t[e];
       *reinterpret_cast<float4 *>(C + x) = make_float4(t[0], t[1], t[2], t[3]);
     } else {
 #pragma unroll
       for (int e = 0; e < 4; e++)
-        if (col + e < p) C[x + e] = EPI && apply ? epi_apply(epi, t[e], x + e) : t[e];
+        if (col + e < p && !((left >> e) & 1u)) C[x + e] = EPI ? epi_apply(epi, t[e], x + e) : t[e];
     }
+    return left;
+  };
+  auto put_again = [&](float *C, int64_t row, int64_t col, float v) {
+    v = sum_in_range(v, RangeArgs{A, B, m, p}, row, col);
+    C[row * p + col] = EPI ? epi_apply(epi, v, row * p + col) : v;
   };
   if (cluster <= 1) {
     // one slice (the epilogue's), or partials that the sum kernel adds
     float *C = out + (int64_t)blockIdx.z * n * p;
+    uint32_t left = 0;
 #pragma unroll
     for (int i = 0; i < TM; i++)
-      put(C, m0 + row0 + 4 * i, n0 + col0, make_float4(acc[i][0], acc[i][1], acc[i][2], acc[i][3]), true);
+      left |= put(C, m0 + row0 + 4 * i, n0 + col0, make_float4(acc[i][0], acc[i][1], acc[i][2], acc[i][3])) << (4 * i);
+    while (RANGE && left != 0) {
+      const int k = __ffs(left) - 1;
+      left &= left - 1;
+      float v = 0.0f;
+#pragma unroll
+      for (int q = 0; q < 4 * TM; q++) v = q == k ? acc[q / 4][q % 4] : v;
+      put_again(C, m0 + row0 + 4 * (k / 4), n0 + col0 + k % 4, v);
+    }
     return;
   }
   __syncthreads();
@@ -534,7 +602,13 @@ simt_ring_kernel(const float *__restrict__ A, const float *__restrict__ B, OutPt
                    : "r"(addr));
       sum = s == 0 ? t : make_float4(sum.x + t.x, sum.y + t.y, sum.z + t.z, sum.w + t.w);
     }
-    put(out, m0 + v / (BN / 4), n0 + (v % (BN / 4)) * 4, sum, true);
+    const int64_t row = m0 + v / (BN / 4), col = n0 + (v % (BN / 4)) * 4;
+    uint32_t left = put(out, row, col, sum);
+    while (RANGE && left != 0) {
+      const int k = __ffs(left) - 1;
+      left &= left - 1;
+      put_again(out, row, col + k, k == 0 ? sum.x : (k == 1 ? sum.y : (k == 2 ? sum.z : sum.w)));
+    }
   }
   // the partials stay until every block of the cluster has read them
   asm volatile("barrier.cluster.arrive.release;\nbarrier.cluster.wait.acquire;" ::: "memory");
@@ -546,7 +620,7 @@ bool f32_vec(const float *A, const float *B, const float *out, int64_t m, int64_
 
 template <int BM, int BN, int TM>
 cudaError_t launch_ring(int64_t n, int64_t m, int64_t p, const float *A, const float *B, float *C, float *part,
-                        int S, int64_t ks, cudaStream_t s, const Epi *epi) {
+                        int S, int64_t ks, cudaStream_t s, const Epi *epi, bool keep_range = false) {
   using R = RingShape<BM, BN, TM>;
   const int64_t gy = ceil_div(n, BM), gx = ceil_div(p, BN);
   if (gy > 65535 || gx > 2147483647LL || S < 1 || S > 65535) return cudaErrorInvalidValue;
@@ -579,17 +653,18 @@ cudaError_t launch_ring(int64_t n, int64_t m, int64_t p, const float *A, const f
     auto launch = [&](auto kernel) {
       return cudaLaunchKernelEx(&cfg, kernel, A, B, out, n, m, p, ks, clustered ? S : 1, early, use ? ep : none);
     };
-    if (use)
-      e = vec ? launch(simt_ring_kernel<BM, BN, TM, true, true>) : launch(simt_ring_kernel<BM, BN, TM, false, true>);
-    else
-      e = vec ? launch(simt_ring_kernel<BM, BN, TM, true, false>) : launch(simt_ring_kernel<BM, BN, TM, false, false>);
+    auto launch_any = [&](auto range) {
+      constexpr bool R = decltype(range)::value;
+      if (use)
+        return vec ? launch(simt_ring_kernel<BM, BN, TM, true, true, R>)
+                   : launch(simt_ring_kernel<BM, BN, TM, false, true, R>);
+      return vec ? launch(simt_ring_kernel<BM, BN, TM, true, false, R>)
+                 : launch(simt_ring_kernel<BM, BN, TM, false, false, R>);
+    };
+    e = keep_range && out == C ? launch_any(std::true_type{}) : launch_any(std::false_type{});
   }
   if (e != cudaSuccess || out == C) return e;
-  TraceScope ts("simt_sum", s);
-  const int64_t np = n * p;
-  if (ceil_div(np, 32) > 2147483647LL) return cudaErrorInvalidValue;
-  return launch_dependent(splitk_sum_kernel<float>, dim3((unsigned)ceil_div(np, 32), 1, 1), s,
-                          static_cast<const float *>(part), S, np, C, static_cast<const int *>(nullptr), ep);
+  return launch_sum(n, m, p, A, B, C, part, S, s, nullptr, ep, keep_range);
 }
 
 // The tile of an FP32 product in S slices of K.  The CUDA cores bound it, so
@@ -659,12 +734,13 @@ bool simt_beats_fused(int64_t n, int64_t m, int64_t p, const SimtPlan &pl) {
 
 cudaError_t launch_simt_splitk_f32(int64_t n, int64_t m, int64_t p, const float *A, const float *B,
                                    float *C, float *part, const SimtPlan &pl, cudaStream_t s,
-                                   const Epi *epi) {
+                                   const Epi *epi, bool keep_range) {
   const int tile = f32_tile(n, p, pl.S, f32_vec(A, B, C, m, p), !pl.wide || pl.S <= kSimtCluster);
-  if (tile == 32) return launch_ring<32, 32, 4>(n, m, p, A, B, C, part, pl.S, pl.ks, s, epi);
-  if (tile == 64) return launch_ring<64, 64, 8>(n, m, p, A, B, C, part, pl.S, pl.ks, s, epi);
+  if (tile == 32) return launch_ring<32, 32, 4>(n, m, p, A, B, C, part, pl.S, pl.ks, s, epi, keep_range);
+  if (tile == 64) return launch_ring<64, 64, 8>(n, m, p, A, B, C, part, pl.S, pl.ks, s, epi, keep_range);
+  // (more than kSimtCluster slices: the sum kernel writes C)
   return launch_splitk<float, kSimtF32BM, kSimtF32BN, kSimtF32BK, 8, 8>(n, m, p, A, B, C, part, pl, s,
-                                                                       "simt_f32", nullptr, epi);
+                                                                       "simt_f32", nullptr, epi, keep_range);
 }
 
 // FP64 products whose 64 x 64 tiles leave the last round of the SMs partly empty
