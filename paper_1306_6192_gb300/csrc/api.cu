@@ -66,20 +66,22 @@ cudaError_t Scratch::reserve(size_t need, cudaStream_t s) {
     want = need;
   }
   bytes = want;
-  return cudaSuccess;
+  return make_words();
+}
+
+cudaError_t Scratch::make_words() {
+  if (words) return cudaSuccess;
+  words_epoch = 0;
+  const cudaError_t e = cudaMalloc(&words, kWords * sizeof(int));
+  if (e == cudaSuccess) return e;
+  cudaGetLastError();
+  words = nullptr;
+  return cudaErrorMemoryAllocation;
 }
 
 cudaError_t Scratch::take_words(size_t counters, cudaStream_t s, int **state, int **clear) {
-  cudaError_t e = cudaSuccess;
-  if (!words) {
-    e = cudaMalloc(&words, kWords * sizeof(int));
-    if (e != cudaSuccess) {
-      cudaGetLastError();
-      words = nullptr;
-      return cudaErrorMemoryAllocation;
-    }
-    words_epoch = 0;
-  }
+  cudaError_t e = make_words();
+  if (e != cudaSuccess) return e;
   if (3 * kStateWords + counters > kWords) return cudaErrorInvalidValue;
   cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
   e = cudaStreamIsCapturing(s, &cap);

@@ -34,6 +34,9 @@ struct Scratch {
   int words_turn = 0;
   uint64_t words_epoch = 0;
   static constexpr size_t kWords = 8 * 1024;
+  // Allocated with the buffer, so that a call whose buffer is there allocates
+  // nothing (it may be captured).
+  cudaError_t make_words();
   // The state words of the next call on one product (zero on the device when
   // its first kernel runs) and those its last kernel clears; `counters` tail
   // counters must be zero, too.
