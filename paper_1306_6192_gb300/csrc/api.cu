@@ -71,38 +71,40 @@ cudaError_t Scratch::reserve(size_t need, cudaStream_t s) {
 
 cudaError_t Scratch::make_words() {
   if (words) return cudaSuccess;
-  words_epoch = 0;
-  const cudaError_t e = cudaMalloc(&words, kWords * sizeof(int));
+  words_clean = false;
+  const cudaError_t e = cudaMalloc(&words, 3 * kSetWords * sizeof(int));
   if (e == cudaSuccess) return e;
   cudaGetLastError();
   words = nullptr;
   return cudaErrorMemoryAllocation;
 }
 
-cudaError_t Scratch::take_words(size_t counters, cudaStream_t s, int **state, int **clear) {
+cudaError_t Scratch::take_words(size_t counters, cudaStream_t s, int **state, ClearWords *clear) {
   cudaError_t e = make_words();
   if (e != cudaSuccess) return e;
-  if (3 * kStateWords + counters > kWords) return cudaErrorInvalidValue;
+  const size_t used = kStateWords + counters;
+  if (used > kSetWords) return cudaErrorInvalidValue;
   cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
   e = cudaStreamIsCapturing(s, &cap);
   if (e != cudaSuccess) return e;
-  const bool captured = cap != cudaStreamCaptureStatusNone;
-  // a launch or a wait that failed may have left words set
-  if (words_epoch != g_ctx.err_epoch) {
-    e = cudaMemsetAsync(words, 0, kWords * sizeof(int), s);
-    if (e != cudaSuccess) return e;
-    if (!captured) words_epoch = g_ctx.err_epoch;
-  }
-  if (captured) {
+  *clear = ClearWords{nullptr, 0};
+  if (cap != cudaStreamCaptureStatusNone) {
     // a replay does not alternate with other calls: a set of its own, cleared
     // ahead of its kernels
-    *state = words + 2 * kStateWords;
-    *clear = nullptr;
-    return cudaMemsetAsync(*state, 0, kStateWords * sizeof(int), s);
+    *state = words + 2 * kSetWords;
+    return cudaMemsetAsync(*state, 0, used * sizeof(int), s);
   }
-  *state = words + words_turn * kStateWords;
+  if (!words_clean) {
+    e = cudaMemsetAsync(words, 0, 2 * kSetWords * sizeof(int), s);
+    if (e != cudaSuccess) return e;
+    words_clean = true;
+    words_used[0] = words_used[1] = 0;
+  }
+  *state = words + words_turn * kSetWords;
+  words_used[words_turn] = (int)used;
   words_turn ^= 1;
-  *clear = words + words_turn * kStateWords;
+  *clear = ClearWords{words + words_turn * kSetWords, words_used[words_turn]};
+  words_used[words_turn] = 0;
   return cudaSuccess;
 }
 
@@ -111,7 +113,6 @@ void Scratch::release() {
   if (words) cudaFree(words);
   words = nullptr;
   words_turn = 0;
-  words_epoch = 0;
   ptr = nullptr;
   bytes = 0;
   stage.release();
@@ -383,8 +384,7 @@ mm_status check_device_flag(cudaStream_t s) {
   if (e != cudaSuccess) return note_cuda(e);
   if (flag != 0) {
     cudaMemset(g_ctx.d_err, 0, sizeof(int));
-    g_ctx.fused_zero_ptr = nullptr;  // an aborted launch may leave counters and words set
-    g_ctx.err_epoch++;
+    g_ctx.fused_zero_ptr = nullptr;  // an aborted fused launch may leave counters set
     return MM_ETIMEOUT;
   }
   return MM_OK;

@@ -26,22 +26,23 @@ struct Scratch {
   void *ptr = nullptr;
   size_t bytes = 0;
   HostStage stage;  // host side of the tables written into this scratch
-  // Words that are zero between calls (calls on one scratch are ordered on one
-  // stream): two sets of kStateWords, used in turn, of which each call clears
-  // the other's in its last kernel, one for captured calls, and the tail
-  // split's counters, which its last parts reset.  Valid while words_epoch is the library's error epoch.
+  // Words that start at zero in a call on one product (calls on one scratch are
+  // ordered on one stream): two sets of kStateWords state words and the tail
+  // split's counters, used in turn.  Each call's last kernel clears what the call
+  // before it used, first of all and whatever became of that call's waits,
+  // so that no call depends on how another one ended.  Captured calls have
+  // a set of their own, which a memset of the graph clears.
+  static constexpr size_t kSetWords = 8 * 1024;
   int *words = nullptr;
+  bool words_clean = false;  // false: new, or a launch failed
   int words_turn = 0;
-  uint64_t words_epoch = 0;
-  static constexpr size_t kWords = 8 * 1024;
+  int words_used[2] = {0, 0};
   // Allocated with the buffer, so that a call whose buffer is there allocates
   // nothing (it may be captured).
   cudaError_t make_words();
-  // The state words of the next call on one product (zero on the device when
-  // its first kernel runs) and those its last kernel clears; `counters` tail
-  // counters must be zero, too.
-  cudaError_t take_words(size_t counters, cudaStream_t s, int **state, int **clear);
-  int *counters() const { return words + 3 * kStateWords; }
+  // The words of the next call on one product (kStateWords, then `counters`; zero
+  // on the device when its first kernel runs) and those its last kernel clears.
+  cudaError_t take_words(size_t counters, cudaStream_t s, int **state, ClearWords *clear);
   // Makes room for `need` bytes; an existing buffer is freed after `s` has
   // drained (its contents are not kept).
   cudaError_t reserve(size_t need, cudaStream_t s);
@@ -81,7 +82,6 @@ struct Ctx {
   Scratch epi_ws;        // the product of an in-place epilogue run as a second pass
   void *fused_zero_ptr = nullptr;  // fused_ws buffer whose leading counters are zero
   size_t fused_zeroed = 0;         //   and how many bytes of them
-  uint64_t err_epoch = 1;  // counts the device-side waits that ran out
   int ozaki_slices = kOzakiDefaultSlices;  // digit slices S of MM_MODE_OZAKI
   int ozaki_gate = 1;                      // accuracy gate of MM_MODE_OZAKI on
   // host-operand pipeline of mm_gemm: copy streams and per-chunk events

@@ -252,6 +252,16 @@ constexpr int kPackUnscaled = 1, kPackFix = 2;
 constexpr int kFlagScaleA = 1, kFlagScaleB = 2;
 // Words of a call on one product that start at zero: its flags, its "any
 // flagged" word, and from kStateHalf on its kTcSplitF16x3 state words.
+struct ClearWords {  // `count` words from `first`, to be set to zero
+  int *first = nullptr;
+  int count = 0;
+};
+#ifdef __CUDACC__
+// By `threads` threads of one block, from number t on.
+__device__ __forceinline__ void clear_words(const ClearWords &w, int t, int threads) {
+  for (int i = t; i < w.count; i += threads) w.first[i] = 0;
+}
+#endif
 constexpr int kStateFlags = 0, kStateAny = 1, kStateHalf = 4, kStateWords = 16;
 // kPackUnscaled: one block per pack tile.  kPackFix: a persistent grid that
 // returns at once unless *any is set, then re-packs the tiles of flagged
@@ -297,18 +307,17 @@ size_t tc_tail_part_bytes(const TcTail &t, int64_t tiles, int bn);
 // device), or nullptr for units c, c + grid, c + 2 grid, ... on CTA c.
 // uniform_only (FP8 with per-block factors): only the tiles whose rows and
 // columns keep one exponent along K (flags in each problem's cnt) run.
-// clear: device words (kStateWords of them) that the launch sets to zero, or
-// nullptr.
+// clear: device words that the launch sets to zero.
 cudaError_t launch_tc(TcKind kind, const ProbTable &tab, int total_units, const int *unit_map,
                       const int *flags,
                       void *pack_base, int64_t pack_rows, const TcConfig &cfg,
                       int *d_err, cudaStream_t s, const int *order = nullptr,
-                      int uniform_only = 0, int *clear = nullptr);
+                      int uniform_only = 0, ClearWords clear = {});
 // The same for kTcSplitF16x3 tables (tc_half.cu; bn = 128).
 cudaError_t launch_tc_half(const ProbTable &tab, int total_units,
                            const int *unit_map, const int *flags, void *pack_base,
                            int64_t pack_rows, int grid, int *d_err, cudaStream_t s,
-                           const int *order, int *clear);
+                           const int *order, ClearWords clear);
 // Tensor map over the pack region viewed as rows of 128 bytes, boxes of bkb
 // (64 or 128) bytes x box_rows rows with the matching swizzle, into `map` (128
 // bytes, 64-byte aligned).

@@ -161,7 +161,7 @@ mm_status mm_gemm_split_static(int64_t n, int64_t m, int64_t p, const float *A, 
                                           : TcConfig{64, 3, grid, ch.bn};
     e = kind == kTcSplitF16x3
             ? launch_tc_half(tab, (int)tiles, nullptr, d_sflag, pack, rows,
-                             tc_launch_grid(cfg, tiles), d_flag, s, nullptr, nullptr)
+                             tc_launch_grid(cfg, tiles), d_flag, s, nullptr, {})
             : launch_tc(kind, tab, (int)tiles, nullptr, d_sflag, pack, rows, cfg, d_flag, s);
   }
   if (e != cudaSuccess) {

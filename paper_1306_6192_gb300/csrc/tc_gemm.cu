@@ -151,7 +151,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmap,
                const __grid_constant__ ProbTable tab, const SplitProb *__restrict__ dev_probs,
                const int *__restrict__ unit_map,
                const int *__restrict__ flags, int total_units, const int *__restrict__ order,
-               int uniform_only, int *clear, int *err) {
+               int uniform_only, ClearWords clear, int *err) {
   using L = TcLayout<BKB, STAGES, KIND, MAXBN>;
   extern __shared__ uint8_t smem_raw[];
   const uint32_t raw = smem_u32(smem_raw);
@@ -197,7 +197,6 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmap,
   const uint32_t tmem_base = *reinterpret_cast<volatile uint32_t *>(tmem_holder);
   // the set-up above may run beside the end of the stream's previous kernel
   pdl_wait();
-  if (clear != nullptr && blockIdx.x == 0 && threadIdx.x < kStateWords) clear[threadIdx.x] = 0;
   // this CTA's work units, the same sequence for every role: the host's list
   // (grid + 1 offsets, then the units), or units c, c + grid, ...
   const int *ulist = order ? order + gridDim.x + 1 : nullptr;
@@ -355,6 +354,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmap,
     int acc = 0;
     uint32_t acc_phase = 0;
     const int et = threadIdx.x - 64;  // over the epilogue warps
+    if (blockIdx.x == 0) clear_words(clear, et, kEpiThreads);  // beside the first tile's MMAs
     const int half = (warp - 2) >> 2;  // which half of the columns
     for (int ui = i_first; ui < i_end; ui += i_step) {
       const int u = ulist ? ulist[ui] : ui;
@@ -417,10 +417,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmap,
         if (et == 0) *last_flag = atomicAdd(pr.cnt + st, 1) == split_s - 1;
         epilogue_sync();
         store = *last_flag != 0;
-        if (store) {
-          __threadfence();
-          if (et == 0) pr.cnt[st] = 0;  // ready for the next launch
-        }
+        if (store) __threadfence();
       }
       for (int c = c_first; c < c_end && store; c += 32) {
         uint32_t v[32];
@@ -635,7 +632,7 @@ namespace {
 template <int BKB, int STAGES, int KIND, int MAXBN, bool ONE = false>
 cudaError_t launch_tc_t(const ProbTable &tab, const int *unit_map, const int *flags, int total_units, void *pack_base, int64_t pack_rows,
                         int grid, int *d_err, cudaStream_t s, const int *order,
-                        int uniform_only, int *clear) {
+                        int uniform_only, ClearWords clear) {
   if constexpr (KIND != kTcE4m3 && !ONE)
     if (tab.dev == nullptr)
       return launch_tc_t<BKB, STAGES, KIND, MAXBN, true>(tab, unit_map, flags, total_units, pack_base, pack_rows,
@@ -769,7 +766,7 @@ size_t tc_tail_bytes(const TcTail &t, int64_t tiles, int bn) {
 cudaError_t launch_tc(TcKind kind, const ProbTable &tab, int total_units, const int *unit_map,
                       const int *flags, void *pack_base, int64_t pack_rows,
                       const TcConfig &cfg, int *d_err, cudaStream_t s, const int *order,
-                      int uniform_only, int *clear) {
+                      int uniform_only, ClearWords clear) {
   if (total_units <= 0) return cudaSuccess;
   if (pack_rows <= 0 || pack_rows > 0x7fffffffLL) return cudaErrorInvalidValue;
   const int grid = tc_launch_grid(cfg, total_units);

@@ -34,6 +34,7 @@
 //   warp 2     decodes the CTA's work units, 32 at a time, into a ring of
 //              descriptors in shared memory, so that no role waits for the
 //              chain unit list -> map -> table -> state words between tiles
+//   warp 3     of the first CTA clears the words of the call before (ctx.h)
 //   warps 4-11 epilogue: warp w reads lane quarter w & 3 and 64 of the 128
 //              columns: both accumulators, their sum, the exact unscaling; the
 //              accumulators go back to the MMAs before anything is stored.
@@ -79,7 +80,7 @@ static_assert(kStageBytes6 <= kStageBytes, "the three-part form fits the stage")
 constexpr int kAccs = 2, kAccCols = 256;
 constexpr int kUnits = 4;                // descriptor ring
 constexpr int kEpiWarps = kHalfSplitCnt, kEpiThreads = 32 * kEpiWarps;
-constexpr int kFirstEpi = 4;             // warp 3 idles: whole warpgroups share registers
+constexpr int kFirstEpi = 4;             // whole warpgroups share registers
 constexpr int kThreads = 32 * kFirstEpi + kEpiThreads;
 constexpr int kEpiRegs = 224, kRoleRegs = 56;
 static_assert(kEpiThreads * kEpiRegs + 128 * kRoleRegs <= kThreads * 168, "registers of the launch");
@@ -143,7 +144,7 @@ __global__ void __launch_bounds__(kThreads, 1)
 tc_half_kernel(const __grid_constant__ CUtensorMap map, const __grid_constant__ CUtensorMap map6,
                const __grid_constant__ CUtensorMap map_d,
                const __grid_constant__ ProbTable tab, const int *__restrict__ unit_map,
-               const int *__restrict__ flags, int total_units, const int *__restrict__ order, int *clear,
+               const int *__restrict__ flags, int total_units, const int *__restrict__ order, ClearWords clear,
                int *err) {
   extern __shared__ uint8_t smem_raw[];
   const uint32_t raw = smem_u32(smem_raw);
@@ -196,7 +197,6 @@ tc_half_kernel(const __grid_constant__ CUtensorMap map, const __grid_constant__ 
   const uint32_t tmem_base = *reinterpret_cast<volatile uint32_t *>(tmem_holder);
   // the set-up above may run beside the end of the stream's previous kernel
   pdl_wait();
-  if (clear != nullptr && blockIdx.x == 0 && threadIdx.x < kStateWords) clear[threadIdx.x] = 0;
 
   if (warp < kFirstEpi) {
     asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kRoleRegs));
@@ -387,6 +387,8 @@ tc_half_kernel(const __grid_constant__ CUtensorMap map, const __grid_constant__ 
           __syncwarp();
         }
       }
+    } else if (blockIdx.x == 0) {
+      clear_words(clear, lane, 32);
     }
   } else {
     // -------------------------------------------------------- epilogue
@@ -509,7 +511,6 @@ tc_half_kernel(const __grid_constant__ CUtensorMap map, const __grid_constant__ 
         store = __shfl_sync(0xffffffffu, last, 0) != 0;
         if (store) {
           __threadfence();
-          if (lane == 0) *cnt = 0;  // ready for the next launch
           // the parts in order 0..split_s-1 (this part's from its registers)
 #pragma unroll
           for (int k = 0; k < 16; k++) {
@@ -662,7 +663,7 @@ tc_half_kernel(const __grid_constant__ CUtensorMap map, const __grid_constant__ 
 cudaError_t launch_tc_half(const ProbTable &tab, int total_units,
                            const int *unit_map, const int *flags, void *pack_base,
                            int64_t pack_rows, int grid, int *d_err, cudaStream_t s,
-                           const int *order, int *clear) {
+                           const int *order, ClearWords clear) {
   // one CTA per SM: the kernel allocates all 512 TMEM columns
   static_assert(2 * Lay::kSmem > 232448, "must not fit twice on one SM");
   static std::once_flag once;

@@ -172,12 +172,13 @@ mm_status run_tc_groups(Scratch &ws, const mm_problem *probs, int count, cudaStr
   // tail counters in words that are zero between calls: nothing to copy or to
   // set ahead of its kernels
   const bool single = ntab == 1;
-  int *state = nullptr, *clear = nullptr;
+  int *state = nullptr;
+  ClearWords clear;
   if (single) {
     SplitProb &sp = all[0];
     if ((e = ws.take_words(tail_cnts, s, &state, &clear)) != cudaSuccess) return note_cuda(e);
     if (sp.hx) sp.hx = state + kStateHalf;
-    if (sp.split_s > 1) sp.cnt = ws.counters();
+    if (sp.split_s > 1) sp.cnt = state + kStateWords;
   }
   SplitProb *d_tab = reinterpret_cast<SplitProb *>(base + tab_off);
   int *d_orders = reinterpret_cast<int *>(base + tab_off + tab_bytes);
@@ -235,7 +236,7 @@ mm_status run_tc_groups(Scratch &ws, const mm_problem *probs, int count, cudaStr
               : launch_tc(G.kind, dt, (int)G.units, tile_map, flags, base, rows, G.cfg, g_ctx.d_err,
                           s, order, 0, clear);
     if (e != cudaSuccess) {
-      ws.words_epoch = 0;  // the words may be left set
+      ws.words_clean = false;
       return note_cuda(e);
     }
   }
