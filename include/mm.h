@@ -368,7 +368,7 @@ mm_status mm_tune_query_tail(int64_t n, int64_t m, int64_t p, int *tiles,
  * through library scratch, the cluster finishing last adding the others in
  * order).  The result does not depend on timing.  *slices = 0: the product
  * takes the packed path (mm_tune_query_tail); MM_MODE_SPLIT_BF16X3 also takes
- * it, in its fp16 form, for m < 2237 with long slices (1024^3), and
+ * it, in its fp16 form, for m < 2237 with slices of eight K blocks (1024^3), and
  * both modes run the smallest of these products as MM_MODE_SIMT.  Grouped calls and serving
  * batches always take the packed path, so a product's bits there equal a
  * grouped call of that product alone; against mm_gemm they agree within the

@@ -344,15 +344,16 @@ mm_status enqueue_gemm(int64_t n, int64_t m, int64_t p, const void *A, const voi
         const SimtPlan spl = simt_plan(false, n, m, p);
         if (simt_beats_fused(n, m, p, spl)) return enqueue_simt_slices(false, n, m, p, A, B, C, spl, s, epi, true);
       }
-      // with m < 2237 the packed form takes long slices: the fused kernel converts
-      // every operand for each of its tiles, about 9 + 4.4 us a K block of a slice.
-      // The data may turn the packed form to six products (magnitudes out of
-      // fp16's range), about 30 + 0.9 us a K block of the whole, so the line lies
-      // where that is no slower.  GB300, us fused / packed / packed with six:
-      // 1024^3 at eight blocks 44.5 / 25.1 / 44.8; 640 x 1280 x 768 39.9 / - / 50.0 and
-      // 512 x 1100 x 900 30.9 / - / 47.2 stay.
-      const int64_t kb = ceil_div(m, 64), slice = fused ? ceil_div(kb, fpl.S) : 0;
-      if (fused && (kind != kTcSplitF16x3 || 44 * slice < 205 + 9 * kb)) {
+      // With m < 2237 the packed form takes the fused plan's longest slices, of eight
+      // K blocks: the fused kernel converts every operand for each of its tiles,
+      // about 4.4 us a block of a slice, and there even the packed form's six
+      // products (magnitudes out of fp16's range, which only the device sees) are
+      // no slower.  GB300, us fused / packed / packed with six: 1024^3, two
+      // slices, 44.5 / 25.5 / 44.7; 896 x 1536 x 896, three, 57.8 / 29.8 / 41.5; 768 x
+      // 1936 x 768, four, 44.5 / 30.9 / 44.5.  Shorter slices stay: 640 x 1280 x 768, of
+      // four blocks, 39.9 / 26.4 / 50.0; 512 x 1100 x 900, of five, 31.0 / 26.3 / 47.2.
+      const bool longest = fused && ceil_div(ceil_div(m, 64), fpl.S) >= kFusedMaxBlocks;
+      if (fused && (kind != kTcSplitF16x3 || !longest)) {
         return run_fused(g_ctx.fused_ws, n, m, p, static_cast<const float *>(A),
                          static_cast<const float *>(B), static_cast<float *>(C), kind, fpl, s, epi);
       }

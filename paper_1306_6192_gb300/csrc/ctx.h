@@ -165,6 +165,7 @@ size_t tail_scratch_bytes(int64_t n, int64_t m, int64_t p, TcKind kind);
 struct FusedPlan {
   int S, Q, cs;
 };
+constexpr int kFusedMaxBlocks = 8;  // K blocks of 64 in the longest slice
 FusedPlan fused_plan(int64_t n, int64_t m, int64_t p, TcKind kind);
 mm_status run_fused(Scratch &ws, int64_t n, int64_t m, int64_t p, const float *A, const float *B,
                     float *C, TcKind kind, const FusedPlan &plan, cudaStream_t s,
