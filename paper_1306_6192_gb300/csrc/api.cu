@@ -298,8 +298,9 @@ static mm_status enqueue_simt_slices(bool f64, int64_t n, int64_t m, int64_t p, 
                                      void *C, const SimtPlan &pl, cudaStream_t s, const Epi *epi,
                                      bool keep_range) {
   void *part = nullptr;
-  if (pl.S > 1) {
-    cudaError_t e = g_ctx.simt_ws.reserve(simt_scratch_bytes(f64, n, m, p), s);
+  const size_t bytes = simt_scratch_bytes(f64, n, m, p);
+  if (bytes > 0) {
+    cudaError_t e = g_ctx.simt_ws.reserve(bytes, s);
     if (e != cudaSuccess) return note_cuda(e);
     part = g_ctx.simt_ws.ptr;
   }

@@ -721,8 +721,9 @@ SimtPlan simt_plan(bool f64, int64_t n, int64_t m, int64_t p) {
 }
 
 size_t simt_scratch_bytes(bool f64, int64_t n, int64_t m, int64_t p) {
+  // (a cluster of blocks adds up to kSimtCluster FP32 slices without scratch)
   const SimtPlan pl = simt_plan(f64, n, m, p);
-  return pl.S > 1 ? (size_t)pl.S * (size_t)(n * p) * (f64 ? 8 : 4) : 0;
+  return pl.S > (f64 ? 1 : kSimtCluster) ? (size_t)pl.S * (size_t)(n * p) * (f64 ? 8 : 4) : 0;
 }
 
 bool simt_beats_fused(int64_t n, int64_t m, int64_t p, const SimtPlan &pl) {

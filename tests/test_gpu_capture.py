@@ -16,11 +16,11 @@ def _pair(seed, n, m, p):
     return dev(synth.uniform_pm1(seed, (n, m))), dev(synth.uniform_pm1(seed + 1, (m, p)))
 
 
-def _capture(mm, n, m, p, A, B, C, stream):
+def _capture(mm, n, m, p, A, B, C, stream, mode=None):
     g = torch.cuda.CUDAGraph(keep_graph=True)
     torch.cuda.synchronize()
     with torch.cuda.graph(g, stream=stream):
-        st = mm.mm_gemm_async(n, m, p, A, B, C, mm.MM_F32, mm.MM_MODE_SPLIT_BF16X3, stream)
+        st = mm.mm_gemm_async(n, m, p, A, B, C, mm.MM_F32, mm.MM_MODE_SPLIT_BF16X3 if mode is None else mode, stream)
     assert st == mm.MM_OK, mm.mm_strerror(st)
     g.instantiate()
     return g
@@ -62,6 +62,27 @@ def test_single_product_after_a_warm_up(mmlib, warm):
         # an eager call between the replays
         assert mm.mm_gemm(n, m, p, A2, B2, C, mm.MM_F32, md) == mm.MM_OK
         assert torch.equal(C, want[1])
+
+
+@pytest.mark.parametrize("shape,first_call", [((256, 256, 256), True), ((64, 1100, 64), True), ((40, 100, 60), True),
+                                              ((64, 16384, 64), False)], ids=lambda v: "x".join(map(str, v)) if isinstance(v, tuple) else None)
+@pytest.mark.parametrize("mode", ["MM_MODE_SIMT", "MM_MODE_SPLIT_BF16X3"])
+def test_small_products_in_a_cluster_need_no_scratch(mmlib, shape, first_call, mode):
+    """Up to eight K slices are added within a cluster: such a product may be the
+    library's first call and captured.  More slices need one call before."""
+    mm, (n, m, p), md = mmlib, shape, getattr(mmlib, mode)
+    A, B = _pair(9907, n, m, p)
+    want, C = torch.empty(n, p, device="cuda"), torch.zeros(n, p, device="cuda")
+    assert mm.mm_gemm(n, m, p, A, B, want, mm.MM_F32, md) == mm.MM_OK  # (loads the kernels, too)
+    mm.mm_shutdown()
+    assert mm.mm_init(device=0) == mm.MM_OK
+    if not first_call:
+        assert mm.mm_gemm(n, m, p, A, B, C, mm.MM_F32, md) == mm.MM_OK
+    g = _capture(mm, n, m, p, A, B, C, torch.cuda.Stream(), md)
+    C.zero_()
+    g.replay()
+    torch.cuda.synchronize()
+    assert torch.equal(C, want)
 
 
 class _Memset(ctypes.Structure):
