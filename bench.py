@@ -441,9 +441,15 @@ def bench_stress(mm, stream, peaks, reps: int = 10):
             gbs = nbytes / (ms * 1e-3) / 1e9
             out["skinny_64x16384x64_" + name] = {"us": ms * 1e3, "gbs": gbs, "frac_hbm": gbs / hbm}
         out["skinny_check_split"] = gpu_check(mm, n, m, p, As[0], Bs[0], Cs[0], mm.MM_F32)
-        _, tiles, sl, ql, csz = mm.mm_tune_query_splitk(n, m, p)
-        out["skinny_split_path"] = ("fused split-K: %d slices in %d clusters of %d" % (sl, ql, csz)
-                                    if sl else "packed")
+        # the kernels that one call of it launches
+        mm.mm_trace_reset()
+        mm.mm_trace_enable(True)
+        gemm(n, m, p, As[0], Bs[0], Cs[0], mm.MM_MODE_SPLIT_BF16X3)
+        mm.check_status(mm.mm_sync(stream), "skinny traced call")
+        mm.mm_trace_enable(False)
+        out["skinny_split_path"] = " + ".join(
+            k for k in ("simt_f32", "simt_sum", "fused_tc", "split_pack", "split_tc") if mm.mm_trace_read(k)[1])
+        mm.mm_trace_reset()
         del As, Bs, Cs
         # 3c: B = diag(d) through the general product (dense flops counted)
         n = 4096
