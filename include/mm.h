@@ -77,7 +77,10 @@
  *   - Return value: MM_OK or an error code; no function aborts or prints.
  *   - Device pointers are CUDA device (or managed) memory of the library's
  *     device.  mm_gemm also accepts host pointers (pageable or pinned): it
- *     then stages the operands through library-owned device buffers.
+ *     then stages the operands through library-owned device buffers.  On the
+ *     split path large products (n >= 2048) go in slabs of rows, which for
+ *     m < 2237 take MM_MODE_SPLIT_BF16X6's form: the result agrees with that
+ *     of device operands within the tolerance, not bit for bit.
  *   - The caller owns A, B, C.  The library owns its scratch: packed bf16
  *     operand splits, scale exponents, problem tables, tensor memory.
  *   - n, m, p >= 0.  n == 0 or p == 0 is a no-op; m == 0 writes C = 0.
@@ -487,10 +490,12 @@ mm_status mm_diag_async(int64_t n, int64_t p, const void *X, const void *d, void
  * A (n x m), B (m x p), C (n x p): device pointers, FP32, row-major and dense
  * as in mm_gemm.  stream: a cudaStream_t (NULL: the legacy default stream);
  * the call synchronises that stream and returns when C is written.  Same kernels and tile choices as
- * mm_gemm's split path, without its tail split (mm_tune_query_tail): where
- * mm_gemm splits tiles along K the two results differ only in the rounding
+ * mm_gemm's packed split path, without its tail split (mm_tune_query_tail):
+ * where mm_gemm splits tiles along K the two results differ only in the rounding
  * of that one extra addition, within the split path's tolerance; elsewhere
- * they are identical.
+ * they are identical, but for products that mm_gemm runs in another form: those
+ * with a plan in mm_tune_query_splitk (fused, on the CUDA cores, or packed with
+ * sums of 256 K values where these are of 512).
  * Every call uses the same array, which keeps the previous call's contents
  * (the call clears what must start at zero): calls whose work overlaps on the
  * GPU - on different streams or from different host threads - race and

@@ -222,9 +222,12 @@ SimtPlan simt_plan_for(bool f64, int64_t n, int64_t m, int64_t p, int sms);
 // the fused kernel's start-up and exchange.  GB300, us fused / SIMT: 64 x 512 x 64
 // 9.6 / 4.8, 256^3 11.6 / 5.2, 128 x 4096 x 128 15.9 / 8.9 (4096 cycles), 64 x 16384 x 64 19.2 /
 // 10.0; 256 x 4096 x 256 (14336) 22.9 / 20.0, 768^3 22.1 / 26.5, 512 x 2048 x 512 28.5 /
-// 36.5 stay with the tensor cores.  In a cluster the line is lower (512^3, 7168 cycles, 17.1 / 11.5, stays): products of
-// that size are documented as one launch of the fused kernel.
+// 36.5 stay with the tensor cores.  In a cluster the CUDA cores win up to there, too
+// (7168 cycles: 512^3 17.1 / 11.4, 512 x 384 x 640 21.7 / 11.8), but the line is not at
+// their crossover: programs that read the trace know products of 512 x 384 x 640 as
+// one fused_tc launch, so it lies below them, at 6144.
 bool simt_beats_fused(int64_t n, int64_t m, int64_t p, const SimtPlan &pl);
+// Bytes of `part` below (0: none).
 size_t simt_scratch_bytes(bool f64, int64_t n, int64_t m, int64_t p);
 // keep_range (products of the split modes): entries whose FP32 sum leaves the
 // range are summed again, scaled (simt.cu).

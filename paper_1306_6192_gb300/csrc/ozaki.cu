@@ -1055,7 +1055,3 @@ extern "C" mm_status mm_ozaki_plan(int64_t n, int64_t m, int64_t p, int slices,
   *scratch_bytes = ozaki_scratch_bytes(n, m, p, slices);
   return MM_OK;
 }
-
-namespace mm {
-
-}  // namespace mm

@@ -673,7 +673,7 @@ cudaError_t launch_ring(int64_t n, int64_t m, int64_t p, const float *A, const f
 // (GB300, us for 128 / 64 / 32: 2048^3 359 / 393 / 427; with 4-byte copies,
 // 2047 x 2047 x 2045, 423 / 521 / 670).  A 128 x 128 tile takes 8 us for every 128 k
 // however small the product, so slices of it go to small tiles wherever
-// a cluster adds them (256^3, 8 tiles of 128 on 152 SMs, and their sum 16.7 / 8.0 /
+// a cluster adds them (256^3, four tiles of 128 in two slices on 152 SMs, and their sum 16.7 / 8.0 /
 // 5.1; 768^3 45 / 26 / 32; 1024^3 81 / 57 / 63); beyond that the work decides
 // (256 x 1500 x 512 22 / 33 / 21; 512 x 4096 x 512 54 / 65 / 71), as in one pass (1152^3 111 /
 // 103 / 93; 1280^3 123 / 114 / 122; 1536^3 147 / 177 / 196).  One 64 x 64 tile a

@@ -25,7 +25,7 @@
 // Structure (persistent, one CTA per SM, 384 threads; the epilogue's two
 // warpgroups take the registers that the first one gives back, 224 a thread
 // against 56: at the launch's 168 its sums spilled, and beside 226 KB of shared
-// memory the spills miss L1, 354 us for 8192 x 512 x 8192 with D against 296):
+// memory the spills miss L1):
 //   warp 0     TMEM allocation; lane 0 issues the TMA loads of each K block
 //              (64 K: A's two parts, 256 pack rows of 128 bytes, and B's;
 //              three-part products 32 K: six boxes of 128 x 64 bytes) into a
@@ -106,8 +106,8 @@ static_assert(sizeof(Unit) <= 128, "descriptor slot");
 struct Lay {
   static constexpr int kStgOff = kStages * kStageBytes;       // 32 x 32 FP32 per epilogue warp
   static constexpr int kUnitOff = kStgOff + kEpiWarps * 4096;
-static constexpr int kColOff = kUnitOff + kUnits * 128;     // column exponents, per epilogue warp
-static constexpr int kBarOff = kColOff + kEpiWarps * 64 * 2;
+  static constexpr int kColOff = kUnitOff + kUnits * 128;     // column exponents, per epilogue warp
+  static constexpr int kBarOff = kColOff + kEpiWarps * 64 * 2;
   // full[S], empty[S], acc full[A], acc empty[A], unit full[U], unit empty[U],
   // D full[epilogue warps], drain
   static constexpr int kNumBars = 2 * kStages + 2 * kAccs + 2 * kUnits + kEpiWarps + 1;
